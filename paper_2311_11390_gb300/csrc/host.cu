@@ -758,7 +758,7 @@ int alif_vanrossum_backward(int64_t rows, int64_t T, const uint32_t *x, const ui
     if (!(dt_ms > 0.0) || !(tau_ms > 0.0)) return fail(ALIF_EINVAL, "DT and tau_R must be > 0");
     if (rows == 0 || t1 == t0) return ALIF_OK;
     if (!x || !y || !f_start || !g_carry || !grad) return fail(ALIF_EINVAL, "NULL pointer");
-    // the kernel keeps one float per 256-step window and warp in shared memory (<= 32 KB)
+    // the kernel keeps one float per tile of 512 spike words in a fixed shared array
     if ((t1 - t0) > (1LL << 19)) return fail(ALIF_EUNSUPPORTED, "chunk longer than 2^19 steps");
     return launch_status(launch_vr_backward(rows, T, x, y, std::exp(-dt_ms / tau_ms), (float)(2.0 * dt_ms / tau_ms),
                                             t0, t1, f_start, g_carry, grad, t1 - t0,
