@@ -12,16 +12,17 @@
 // steps follow from it.  Inside a word every value is an 8-step chain from a zero start plus an
 // exact power times the value entering those 8 steps, so a rounded decay is never compounded over
 // more than 8 steps.
-// What bounds it: the gradient's writes (4 B per step; the bits are 1/16 of that), with about 15
-// thread instructions per step behind them.  A warp per row walking 256-step windows, as before,
-// left 1024 rows x 400000 steps to 1024 warps that each waited for two spike words per window:
-// forward 0.92 ms and gradient 2.05 ms.
+// What bounds it: the gradient's writes (4 B per step, 0.24 ms for 1024 rows x 400000 steps; the
+// bits are 1/16 of that) and the instructions of the word's chains and scans between the barriers.
+// At that size: forward 0.14 ms, gradient 0.44 ms.  A warp per row walking 256-step windows left it
+// to 1024 warps that each waited for two spike words per window: 0.92 and 2.05 ms.
 #include "common.cuh"
 
 namespace alif {
 namespace vr {
 
 constexpr int E = 8, SUB = 4, WORD = 32;  // a word is SUB chains of E steps
+constexpr int LDS_ROW = WORD + 4;             // floats per staged word: 16-byte rows, no bank conflicts
 constexpr int TH_MAX = 512;               // words per tile
 constexpr long long MAX_ROWS = 1 << 30;   // rows (CTAs) per launch
 constexpr int MAX_TILES = (1 << 19) / WORD / TH_MAX;  // tiles of the longest gradient call
@@ -88,33 +89,53 @@ __device__ __forceinline__ float tile_scan(float e, float carry, const Tables &t
     return fmaf(REV ? tb.ldn : tb.lup, in, excl);
 }
 
-// f of a word's 32 steps from a zero start at each 8-step chain (loc) and the chains' ends joined:
-// the word's contribution to its end.
-__device__ __forceinline__ float word_local(uint32_t xw, uint32_t yw, const Tables &tb, float (&loc)[WORD]) {
-    float end = 0.0f;
-#pragma unroll
-    for (int j = 0; j < SUB; ++j) {
+// lut[m]: the 8 values of f after the spikes in the bits of byte m, from a zero start.  The
+// filter is linear, so a word's chains are two look-ups per 8 steps (x without y, y without x;
+// mostly entry 0, a broadcast) and a packed subtraction, against 7 instructions per step to turn
+// each pair of bits into +-1 and carry it.
+struct __align__(16) Chain {
+    float2 v[E / 2];
+};
+
+__device__ __forceinline__ void make_lut(Chain *lut, const Tables &tb) {
+    for (int m = threadIdx.x; m < 256; m += blockDim.x) {
         float f = 0.0f;
 #pragma unroll
         for (int k = 0; k < E; ++k) {
-            const int s = E * j + k;
-            const float dv = ((xw >> s) & 1u ? 1.0f : 0.0f) - ((yw >> s) & 1u ? 1.0f : 0.0f);
-            f = fmaf(tb.pw[1], f, dv);
-            loc[s] = f;
+            f = fmaf(tb.pw[1], f, (m >> k) & 1 ? 1.0f : 0.0f);
+            (k & 1 ? lut[m].v[k / 2].y : lut[m].v[k / 2].x) = f;
         }
-        end = fmaf(tb.pw[E], end, f);
+    }
+    __syncthreads();
+}
+
+// f of a word's 32 steps from a zero start at each 8-step chain; returns the chains' ends joined:
+// the word's contribution to its end.
+__device__ __forceinline__ float word_local(uint32_t xw, uint32_t yw, const Tables &tb, const Chain *lut,
+                                            float2 (&f)[WORD / 2]) {
+    const uint32_t up = xw & ~yw, dn = yw & ~xw;
+    float end = 0.0f;
+#pragma unroll
+    for (int j = 0; j < SUB; ++j) {
+        const Chain a = lut[(up >> (8 * j)) & 255u], b = lut[(dn >> (8 * j)) & 255u];
+#pragma unroll
+        for (int k = 0; k < E / 2; ++k) f[E / 2 * j + k] = __ffma2_rn(make_float2(-1.0f, -1.0f), b.v[k], a.v[k]);
+        end = fmaf(tb.pw[E], end, f[E / 2 * j + E / 2 - 1].y);
     }
     return end;
 }
 
 // The word's f values from the value entering it.
-__device__ __forceinline__ void word_apply(float fin, const Tables &tb, float (&f)[WORD]) {
+__device__ __forceinline__ void word_apply(float fin, const Tables &tb, float2 (&f)[WORD / 2]) {
     float s = fin;
 #pragma unroll
     for (int j = 0; j < SUB; ++j) {
-        const float next = fmaf(tb.pw[E], s, f[E * j + E - 1]);
+        const float next = fmaf(tb.pw[E], s, f[E / 2 * j + E / 2 - 1].y);
 #pragma unroll
-        for (int k = 0; k < E; ++k) f[E * j + k] = fmaf(tb.pw[k + 1], s, f[E * j + k]);
+        for (int k = 0; k < E / 2; ++k) {
+            float2 &v = f[E / 2 * j + k];
+            v = __ffma2_rn(make_float2(tb.pw[2 * k + 1], tb.pw[2 * k + 2]), make_float2(s, s), v);
+        }
         s = next;
     }
 }
@@ -128,11 +149,13 @@ __global__ void __launch_bounds__(TH_MAX, 2) vr_forward_kernel(long long T, cons
                                                             const uint32_t *__restrict__ y, double dec, double scale,
                                                             long long chunk, long long nchunk, float *f_ckpt,
                                                             float *loss) {
+    __shared__ Chain lut[256];
     __shared__ float ws[2][16];
     __shared__ df sums[16];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
     const long long r = blockIdx.x;
     const Tables tb = make_tables(dec, lane);
+    make_lut(lut, tb);
     const long long nwords = (T + 31) / 32;
     const uint32_t *xb = x + r * nwords, *yb = y + r * nwords;
     const long long ntile = (nwords + blockDim.x - 1) / blockDim.x;
@@ -145,20 +168,22 @@ __global__ void __launch_bounds__(TH_MAX, 2) vr_forward_kernel(long long T, cons
         const long long qn = q + blockDim.x;
         xn = qn < nwords ? __ldg(xb + qn) : 0u;  // the next tile's words, in flight during this one
         yn = qn < nwords ? __ldg(yb + qn) : 0u;
-        float f[WORD];
-        const float e = word_local(xw, yw, tb, f);
+        float2 f[WORD / 2];
+        const float e = word_local(xw, yw, tb, lut, f);
         const float fin = tile_scan<false>(e, carry, tb, ws[i & 1], lane, warp, nw, &carry);
         if (f_ckpt && q < nwords && (32 * q) % chunk == 0) f_ckpt[r * nchunk + 32 * q / chunk] = fin;
         word_apply(fin, tb, f);
-        float s[SUB];
+        float2 s[2] = {};
+        if (valid != ~0u) {
 #pragma unroll
-        for (int j = 0; j < SUB; ++j) {
-            s[j] = 0.0f;
-#pragma unroll
-            for (int k = 0; k < E; ++k)
-                if ((valid >> (E * j + k)) & 1u) s[j] = fmaf(f[E * j + k], f[E * j + k], s[j]);
+            for (int k = 0; k < WORD / 2; ++k) {
+                f[k].x = (valid >> (2 * k)) & 1u ? f[k].x : 0.0f;
+                f[k].y = (valid >> (2 * k + 1)) & 1u ? f[k].y : 0.0f;
+            }
         }
-        acc = df_add(acc, df{(s[0] + s[1]) + (s[2] + s[3]), 0.0f});
+#pragma unroll
+        for (int k = 0; k < WORD / 2; ++k) s[k & 1] = __ffma2_rn(f[k], f[k], s[k & 1]);
+        acc = df_add(acc, df{(s[0].x + s[0].y) + (s[1].x + s[1].y), 0.0f});
     }
 #pragma unroll
     for (int off = 16; off; off >>= 1) {
@@ -175,31 +200,41 @@ __global__ void __launch_bounds__(TH_MAX, 2) vr_forward_kernel(long long T, cons
 
 // Gradient for steps [t0, t1) (t0 a multiple of 256 and of the chunk start):
 // grad[r, t - t0] = (2 DT / tau_R) g[t], g carried from t1 in g_carry (updated).
-// VEC: floats per store (8 where grad rows keep 32 bytes: whole sectors from each lane).
-template <int VEC>
+// VEC: gradient rows keep 16 bytes, so a warp passes its words through shared memory and writes
+// whole lines (0.50 ms at 1024 x 400000; 0.59 with each lane storing its own 128 bytes; 0.44 with
+// the words loaded a tile ahead).
+template <bool VEC>
 __global__ void __launch_bounds__(TH_MAX, 2) vr_backward_kernel(long long nwords, const uint32_t *__restrict__ x,
                                                              const uint32_t *__restrict__ y, double dec, float gscale,
                                                              long long t0, long long t1,
                                                              const float *__restrict__ f_start, float *g_carry,
                                                              float *grad, long long ldg) {
+    __shared__ Chain lut[256];
     __shared__ float ws[2][16];
     __shared__ float ftile[MAX_TILES];  // f entering each tile
+    extern __shared__ __align__(16) float stages[];  // [warps][32][LDS_ROW]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5, th = blockDim.x;
     const long long r = blockIdx.x;
     const Tables tb = make_tables(dec, lane);
+    make_lut(lut, tb);
+    float *stage = stages + warp * 32 * LDS_ROW;
     const uint32_t *xb = x + r * nwords + (t0 >> 5), *yb = y + r * nwords + (t0 >> 5);
     const int steps = (int)(t1 - t0), nq = (steps + 31) / 32, ntile = (nq + th - 1) / th;
+    // a tile's words are loaded while the tile before it in the loop is resolved
+    uint32_t xn = tid < nq ? __ldg(xb + tid) : 0u, yn = tid < nq ? __ldg(yb + tid) : 0u;
     int par = 0;
     float carry = f_start[r];
     for (int i = 0; i < ntile; ++i) {
         if (tid == 0) ftile[i] = carry;
-        if (i + 1 == ntile) break;
-        const int q = i * th + tid;  // every tile but the last is full
-        const uint32_t xw = __ldg(xb + q), yw = __ldg(yb + q);
+        if (i + 1 == ntile) break;  // xn, yn: the last tile's, where the reverse loop starts
+        const int qn = (i + 1) * th + tid;  // every tile but the last is full
+        const uint32_t xw = xn, yw = yn;
+        xn = qn < nq ? __ldg(xb + qn) : 0u;
+        yn = qn < nq ? __ldg(yb + qn) : 0u;
         float e = 0.0f;
         if (xw != yw) {
-            float f[WORD];
-            e = word_local(xw, yw, tb, f);
+            float2 f[WORD / 2];
+            e = word_local(xw, yw, tb, lut, f);
         }
         tile_scan<false>(e, carry, tb, ws[par], lane, warp, nw, &carry);
         par ^= 1;
@@ -210,12 +245,23 @@ __global__ void __launch_bounds__(TH_MAX, 2) vr_backward_kernel(long long nwords
     for (int i = ntile - 1; i >= 0; --i) {
         const int q = i * th + tid, cnt = steps - 32 * q;  // steps of this word (may be <= 0)
         const uint32_t valid = below(cnt);
-        const uint32_t xw = q < nq ? __ldg(xb + q) & valid : 0u, yw = q < nq ? __ldg(yb + q) & valid : 0u;
-        float f[WORD], unused;
-        const float e = word_local(xw, yw, tb, f);
+        const uint32_t xw = xn & valid, yw = yn & valid;
+        if (i > 0) {
+            xn = __ldg(xb + q - th);
+            yn = __ldg(yb + q - th);
+        }
+        float2 f2[WORD / 2];
+        float unused;
+        const float e = word_local(xw, yw, tb, lut, f2);
         const float fin = tile_scan<false>(e, ftile[i], tb, ws[par], lane, warp, nw, &unused);
         par ^= 1;
-        word_apply(fin, tb, f);
+        word_apply(fin, tb, f2);
+        float f[WORD];
+#pragma unroll
+        for (int k = 0; k < WORD / 2; ++k) {
+            f[2 * k] = f2[k].x;
+            f[2 * k + 1] = f2[k].y;
+        }
         // the word that holds step t1 - 1 takes the carry of step t1 there; nothing passes through
         // it from later words
         const bool last = q == nq - 1;
@@ -240,31 +286,33 @@ __global__ void __launch_bounds__(TH_MAX, 2) vr_backward_kernel(long long nwords
         for (int j = SUB - 1; j >= 0; --j) {
             const float next = fmaf(tb.pw[E], s, f[E * j]);
 #pragma unroll
-            for (int k = 0; k < E; ++k) f[E * j + k] = fmaf(tb.pw[E - k], s, f[E * j + k]);
-            s = next;
-        }
-        if (q == 0) g_carry[r] = f[0];
-        float *go = grad + r * ldg + 32LL * q;
-        if (VEC > 1 && cnt >= WORD) {
-#pragma unroll
-            for (int k = 0; k < WORD; k += 8) {
-                if (VEC == 8) {
-                    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(go + k),
-                                 "f"(gscale * f[k]), "f"(gscale * f[k + 1]), "f"(gscale * f[k + 2]),
-                                 "f"(gscale * f[k + 3]), "f"(gscale * f[k + 4]), "f"(gscale * f[k + 5]),
-                                 "f"(gscale * f[k + 6]), "f"(gscale * f[k + 7])
-                                 : "memory");
-                } else {
-#pragma unroll
-                    for (int m = k; m < k + 8; m += 4)
-                        *reinterpret_cast<float4 *>(go + m) = make_float4(
-                            gscale * f[m], gscale * f[m + 1], gscale * f[m + 2], gscale * f[m + 3]);
-                }
+            for (int k = 0; k < E; k += 2) {
+                const float2 v = __fmul2_rn(
+                    make_float2(gscale, gscale),
+                    __ffma2_rn(make_float2(tb.pw[E - k], tb.pw[E - k - 1]), make_float2(s, s),
+                               make_float2(f[E * j + k], f[E * j + k + 1])));
+                f[E * j + k] = v.x;
+                f[E * j + k + 1] = v.y;
             }
+            s = next;
+            if (j == 0 && q == 0) g_carry[r] = next;
+        }
+        float *go = grad + r * ldg + 32LL * q;
+        if (VEC && __all_sync(FULL, cnt >= WORD)) {  // the warp's 32 words: 4 KB, written line by line
+#pragma unroll
+            for (int k = 0; k < WORD; k += 4)
+                *reinterpret_cast<float4 *>(stage + lane * LDS_ROW + k) = make_float4(f[k], f[k + 1], f[k + 2], f[k + 3]);
+            __syncwarp();
+            float *gw = go - 32 * lane + 4 * lane;
+#pragma unroll
+            for (int k = 0; k < WORD / 4; ++k)
+                *reinterpret_cast<float4 *>(gw + 128 * k) =
+                    *reinterpret_cast<const float4 *>(stage + (4 * k + (lane >> 3)) * LDS_ROW + 4 * (lane & 7));
+            __syncwarp();
         } else {
 #pragma unroll
             for (int k = 0; k < WORD; ++k)
-                if (k < cnt) go[k] = gscale * f[k];
+                if (k < cnt) go[k] = f[k];
         }
     }
 }
@@ -296,13 +344,16 @@ int launch_vr_backward(long long rows, long long T, const uint32_t *x, const uin
                        cudaStream_t st) {
     const long long nwords = (T + 31) / 32;
     const unsigned th = vr::threads_for((t1 - t0 + 31) / 32);
-    const uintptr_t ga = reinterpret_cast<uintptr_t>(grad);
-    const auto kernel = (ldg % 8 == 0 && ga % 32 == 0)   ? vr::vr_backward_kernel<8>
-                        : (ldg % 4 == 0 && ga % 16 == 0) ? vr::vr_backward_kernel<4>
-                                                         : vr::vr_backward_kernel<1>;
+    const bool vec = ldg % 4 == 0 && reinterpret_cast<uintptr_t>(grad) % 16 == 0;
+    const auto kernel = vec ? vr::vr_backward_kernel<true> : vr::vr_backward_kernel<false>;
+    const size_t smem = vec ? (size_t)th * vr::LDS_ROW * sizeof(float) : 0;
+    if (smem > 32768) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return (int)e;
+    }
     for (long long r = 0; r < rows; r += vr::MAX_ROWS) {
         const unsigned n = (unsigned)(rows - r < vr::MAX_ROWS ? rows - r : vr::MAX_ROWS);
-        kernel<<<n, th, 0, st>>>(nwords, x + r * nwords, y + r * nwords, dec, gscale, t0, t1, f_start + r, g_carry + r,
+        kernel<<<n, th, smem, st>>>(nwords, x + r * nwords, y + r * nwords, dec, gscale, t0, t1, f_start + r, g_carry + r,
                                  grad + r * ldg, ldg);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return (int)e;
