@@ -141,19 +141,29 @@ int launch_status(int rc, const char *what) {
     return ALIF_OK;
 }
 
-__global__ void reduce_params_kernel(const float *part, float *out, long long B, long long N) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    df acc[ALIF_NUM_PARAM_GRADS];
-#pragma unroll
-    for (int k = 0; k < ALIF_NUM_PARAM_GRADS; ++k) acc[k] = df{0.0f, 0.0f};
-    for (long long b = 0; b < B; ++b) {  // fixed order: deterministic
-        const float *q = part + (b * N + i) * (2 * ALIF_NUM_PARAM_GRADS);
-#pragma unroll
-        for (int k = 0; k < ALIF_NUM_PARAM_GRADS; ++k) acc[k] = df_add(acc[k], df{q[2 * k], q[2 * k + 1]});
+// Sums of the per-row parameter partials over the batch.  Element e = 5 i + k (neuron i, parameter
+// k) is thread x of a 32-element column block, so a warp reads 256 consecutive bytes of a batch
+// element; the batch is split over blockDim.y threads (every blockDim.y-th element each, then a
+// fixed tree: deterministic).  Bound by latency: one thread per neuron walking the batch with five
+// serial double-single additions took 76 us at B = 128, N = 256 (two blocks on the chip).
+constexpr int REDUCE_MAX_Y = 32;
+
+__global__ void reduce_params_kernel(const float *__restrict__ part, float *out, long long B, long long N) {
+    __shared__ df sums[REDUCE_MAX_Y][33];
+    const long long ne = N * ALIF_NUM_PARAM_GRADS;
+    const long long e = (long long)blockIdx.x * 32 + threadIdx.x;
+    df acc{0.0f, 0.0f};
+    if (e < ne)
+        for (long long b = threadIdx.y; b < B; b += blockDim.y) {
+            const float *q = part + 2 * (b * ne + e);
+            acc = df_add(acc, df{q[0], q[1]});
+        }
+    for (int half = blockDim.y >> 1; half; half >>= 1) {  // blockDim.y is a power of two
+        if (threadIdx.y >= half && threadIdx.y < 2 * half) sums[threadIdx.y][threadIdx.x] = acc;
+        __syncthreads();
+        if (threadIdx.y < half) acc = df_add(acc, sums[threadIdx.y + half][threadIdx.x]);
     }
-#pragma unroll
-    for (int k = 0; k < ALIF_NUM_PARAM_GRADS; ++k) out[k * N + i] = acc[k].hi + acc[k].lo;
+    if (threadIdx.y == 0 && e < ne) out[(e % ALIF_NUM_PARAM_GRADS) * N + e / ALIF_NUM_PARAM_GRADS] = acc.hi + acc.lo;
 }
 
 __global__ void copy_state_kernel(const AlifState *init, AlifState *fin, long long rows) {
@@ -166,11 +176,13 @@ __global__ void copy_state_kernel(const AlifState *init, AlifState *fin, long lo
 
 int reduce_params(const float *part, float *out, long long B, long long N, cudaStream_t st) {
     if (N == 0) return ALIF_OK;
-    const int threads = 128;
+    unsigned y = 1;
+    while (y < B && y < REDUCE_MAX_Y) y *= 2;
     // the launch's own status (cudaGetLastError could report an earlier, unrelated failure)
     void *args[] = {&part, &out, &B, &N};
     const cudaError_t e = cudaLaunchKernel((const void *)reduce_params_kernel,
-                                           dim3((unsigned)((N + threads - 1) / threads)), dim3(threads), args, 0, st);
+                                           dim3((unsigned)((N * ALIF_NUM_PARAM_GRADS + 31) / 32)), dim3(32, y), args,
+                                           0, st);
     return e == cudaSuccess ? ALIF_OK : cuda_fail(e, "reduce_params_kernel");
 }
 
