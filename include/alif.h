@@ -439,6 +439,19 @@ int syn_project(int64_t B, int64_t Nin, int64_t N, int64_t T,
                 const uint16_t *W_hi, const uint16_t *W_lo, int64_t ldw,
                 const uint32_t *S_in, const float *bias, float *I, void *stream);
 
+/* syn_project() with a workspace for the event lists of sparse rasters.  256-step tiles whose
+ * chunks of 32 steps are sparse enough (at Nin = 1000 about 12 active inputs per step) are summed over
+ * the active inputs only, with the weights W_hi + W_lo in FP32, inputs ascending and the bias last:
+ * within (k + 1) 2^-24 (|bias_i| + sum_j |W_ij| S_j) of the exact sum of W_hi + W_lo for k active
+ * inputs.  The other tiles run on the tensor cores as in syn_project().  A weight that is not finite
+ * makes its neuron's currents NaN in both.  The workspace (256-byte aligned) holds
+ * syn_project_workspace_size() bytes; that is 0 for sizes the tensor cores always take (small
+ * products, Nin > 1024), and with workspace = NULL every tile runs there. */
+size_t syn_project_workspace_size(int64_t B, int64_t Nin, int64_t N, int64_t T);
+int syn_project_ws(int64_t B, int64_t Nin, int64_t N, int64_t T, const uint16_t *W_hi, const uint16_t *W_lo,
+                   int64_t ldw, const uint32_t *S_in, const float *bias, float *I, void *workspace,
+                   size_t workspace_bytes, void *stream);
+
 /* Workspace bytes syn_project_backward() needs: the per-batch-element partial
  * sums of grad_W / grad_bias (reduced in a fixed order) and the two BF16 terms
  * of W^T used for grad_Sin. */
@@ -475,6 +488,14 @@ int syn_project_backward(int64_t B, int64_t Nin, int64_t N, int64_t T, const flo
  * Device pointers; asynchronous on `stream`. */
 int syn_project_events(int64_t B, int64_t Nin, int64_t N, int64_t T, const float *W_t,
                        const uint32_t *S_in, const float *bias, float *I, void *stream);
+
+/* syn_project_events() with a workspace (256-byte aligned, syn_project_events_workspace_size()
+ * bytes; 0 where it is not used) that holds each chunk's event list, built once for all neurons.
+ * Same sums, inputs ascending, the bias last; tiles too dense for the lists, and calls with
+ * workspace = NULL, build them per CTA. */
+size_t syn_project_events_workspace_size(int64_t B, int64_t Nin, int64_t N, int64_t T);
+int syn_project_events_ws(int64_t B, int64_t Nin, int64_t N, int64_t T, const float *W_t, const uint32_t *S_in,
+                          const float *bias, float *I, void *workspace, size_t workspace_bytes, void *stream);
 
 /* W [N, Nin] -> W_t [Nin, N] (the layout syn_project_events reads). */
 int syn_transpose_weights(const float *W, int64_t N, int64_t Nin, float *W_t, void *stream);

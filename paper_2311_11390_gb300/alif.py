@@ -59,6 +59,8 @@ def lib():
                               ctypes.c_int),
         "syn_split_bf16": ([P, i64, i64, i64, P, P, P], ctypes.c_int),
         "syn_project": ([i64, i64, i64, i64, P, P, i64, P, P, P, P], ctypes.c_int),
+        "syn_project_workspace_size": ([i64, i64, i64, i64], sz),
+        "syn_project_ws": ([i64, i64, i64, i64, P, P, i64, P, P, P, P, sz, P], ctypes.c_int),
         "syn_project_backward_workspace_size": ([i64, i64, i64], sz),
         "syn_project_backward": ([i64, i64, i64, i64, P, P, P, P, P, P, P, sz, P], ctypes.c_int),
         "alif_unpack_spikes": ([i64, i64, P, P, P], ctypes.c_int),
@@ -66,6 +68,8 @@ def lib():
         "alif_pack_spikes": ([i64, i64, P, P, P], ctypes.c_int),
         "syn_transpose_weights": ([P, i64, i64, P, P], ctypes.c_int),
         "syn_project_events": ([i64, i64, i64, i64, P, P, P, P, P], ctypes.c_int),
+        "syn_project_events_workspace_size": ([i64, i64, i64, i64], sz),
+        "syn_project_events_ws": ([i64, i64, i64, i64, P, P, P, P, P, sz, P], ctypes.c_int),
         "alif_forward_recurrent": ([i64, i64, i64, P, P, P, f64, f64, P, P, P, P, P, P], ctypes.c_int),
         "alif_delay_spikes": ([i64, i64, i64, i64, P, P, P], ctypes.c_int),
         "alif_readout_forward": ([i64, i64, i64, i64, P, P, P, P, f32, P, P, P], ctypes.c_int),
@@ -426,7 +430,8 @@ def split_bf16(W: torch.Tensor, ldw: int | None = None):
 
 def syn_project(S_words: torch.Tensor, W_hi: torch.Tensor, W_lo: torch.Tensor, bias=None, Nin=None, T=None,
                 out=None):
-    """I[b, i, t] = bias_i + sum_j W[i, j] S[b, j, t] on the tensor cores.
+    """I[b, i, t] = bias_i + sum_j W[i, j] S[b, j, t]: sums over the active inputs where the raster is
+    sparse, the tensor cores elsewhere.
     S_words: int32 [B, Nin, ceil(T/32)] spike bits; W_hi/W_lo from split_bf16."""
     B, Nin_s, nw = S_words.shape
     Nin = Nin_s if Nin is None else Nin
@@ -434,8 +439,11 @@ def syn_project(S_words: torch.Tensor, W_hi: torch.Tensor, W_lo: torch.Tensor, b
     N, ldw = W_hi.shape
     if out is None:
         out = torch.empty((B, N, T), dtype=torch.float32, device=S_words.device)
-    _check(lib().syn_project(B, Nin, N, T, _ptr(W_hi), _ptr(W_lo), ldw, _ptr(S_words), _ptr(bias), _ptr(out),
-                             _stream(S_words.device)), "syn_project")
+    L = lib()
+    wsz = int(L.syn_project_workspace_size(B, Nin, N, T))
+    ws = torch.empty(wsz, dtype=torch.uint8, device=S_words.device) if wsz else None
+    _check(L.syn_project_ws(B, Nin, N, T, _ptr(W_hi), _ptr(W_lo), ldw, _ptr(S_words), _ptr(bias), _ptr(out),
+                            _ptr(ws), wsz, _stream(S_words.device)), "syn_project")
     return out
 
 
@@ -560,6 +568,9 @@ def syn_project_events(S_words: torch.Tensor, W_t: torch.Tensor, bias=None, Nin=
     N = W_t.shape[1]
     if out is None:
         out = torch.empty((B, N, T), dtype=torch.float32, device=S_words.device)
-    _check(lib().syn_project_events(B, Nin, N, T, _ptr(W_t), _ptr(S_words), _ptr(bias), _ptr(out),
-                                    _stream(S_words.device)), "syn_project_events")
+    L = lib()
+    wsz = int(L.syn_project_events_workspace_size(B, Nin, N, T))
+    ws = torch.empty(wsz, dtype=torch.uint8, device=S_words.device) if wsz else None
+    _check(L.syn_project_events_ws(B, Nin, N, T, _ptr(W_t), _ptr(S_words), _ptr(bias), _ptr(out), _ptr(ws), wsz,
+                                   _stream(S_words.device)), "syn_project_events")
     return out

@@ -51,7 +51,11 @@ int launch_split_pad(const float *W, long long N, long long Nin, long long ldw, 
                      cudaStream_t stream);
 int launch_syn_project(long long B, long long Nin, long long N, long long T, const uint16_t *W_hi,
                        const uint16_t *W_lo, long long ldw, const uint32_t *S, const float *bias, float *I,
-                       int *status, cudaStream_t stream);
+                       const uint32_t *dense, int *status, cudaStream_t stream);
+size_t syn_sparse_ws(long long B, long long Nin, long long N, long long T, bool split);
+int launch_syn_sparse(long long B, long long Nin, long long N, long long T, const float *Wt, const uint16_t *hi,
+                      const uint16_t *lo, long long ldw, const uint32_t *S, const float *bias, float *I, void *work,
+                      const uint32_t **dense, cudaStream_t st);
 
 size_t syn_project_backward_ws(long long B, long long N, long long Nin);
 int launch_syn_project_backward(long long B, long long Nin, long long N, long long T, const float *W,
@@ -68,7 +72,7 @@ int launch_cross_entropy(long long B, long long C, const float *o, const int32_t
 int launch_pack_spikes(long long rows, long long T, const float *S, uint32_t *words, cudaStream_t st);
 int launch_transpose_weights(const float *W, long long N, long long Nin, float *Wt, cudaStream_t st);
 int launch_syn_project_events(long long B, long long Nin, long long N, long long T, const float *Wt,
-                              const uint32_t *S, const float *bias, float *I, cudaStream_t st);
+                              const uint32_t *S, const float *bias, float *I, const uint32_t *dense, cudaStream_t st);
 int launch_vr_forward(long long rows, long long T, const uint32_t *x, const uint32_t *y, double dec, double scale,
                       long long chunk, float *f_ckpt, float *loss, cudaStream_t st);
 int launch_vr_backward(long long rows, long long T, const uint32_t *x, const uint32_t *y, double dec, float gscale,
@@ -652,8 +656,18 @@ __global__ void bias_fill_kernel(const float *bias, float *I, long long N, long 
         I[k] = bias ? bias[(k / T) % N] : 0.0f;
 }
 
+size_t syn_project_workspace_size(int64_t B, int64_t Nin, int64_t N, int64_t T) {
+    return syn_sparse_ws(B, Nin, N, T, true);
+}
+
 int syn_project(int64_t B, int64_t Nin, int64_t N, int64_t T, const uint16_t *W_hi, const uint16_t *W_lo,
                 int64_t ldw, const uint32_t *S_in, const float *bias, float *I, void *stream) {
+    return syn_project_ws(B, Nin, N, T, W_hi, W_lo, ldw, S_in, bias, I, nullptr, 0, stream);
+}
+
+int syn_project_ws(int64_t B, int64_t Nin, int64_t N, int64_t T, const uint16_t *W_hi, const uint16_t *W_lo,
+                   int64_t ldw, const uint32_t *S_in, const float *bias, float *I, void *workspace,
+                   size_t workspace_bytes, void *stream) {
     int rc = check_shape(B, N, T);
     if (rc) return rc;
     if (Nin < 0 || ldw < Nin || ldw % ALIF_PROJ_K_ALIGN != 0)
@@ -675,7 +689,15 @@ int syn_project(int64_t B, int64_t Nin, int64_t N, int64_t T, const uint16_t *W_
     Symbols *s = nullptr;
     rc = symbols(&s);
     if (rc) return rc;
-    const int r = launch_syn_project(B, Nin, N, T, W_hi, W_lo, ldw, S_in, bias, I, s->status, st);
+    const uint32_t *dense = nullptr;
+    const size_t need = workspace ? syn_sparse_ws(B, Nin, N, T, true) : 0;
+    if (need) {
+        if (!aligned(workspace, 256)) return fail(ALIF_ESHAPE, "workspace must be 256-byte aligned");
+        if (workspace_bytes < need) return fail(ALIF_EWORKSPACE, "workspace too small: need %zu bytes", need);
+        const int e = launch_syn_sparse(B, Nin, N, T, nullptr, W_hi, W_lo, ldw, S_in, bias, I, workspace, &dense, st);
+        if (e) return launch_status(e, "syn_project sparse launch");
+    }
+    const int r = launch_syn_project(B, Nin, N, T, W_hi, W_lo, ldw, S_in, bias, I, dense, s->status, st);
     if (r < 0) return fail(ALIF_EUNSUPPORTED, "cuTensorMapEncodeTiled unavailable or rejected the weights");
     return launch_status(r, "syn_project launch");
 }
@@ -842,20 +864,34 @@ int syn_transpose_weights(const float *W, int64_t N, int64_t Nin, float *W_t, vo
                          "transpose_kernel");
 }
 
+size_t syn_project_events_workspace_size(int64_t B, int64_t Nin, int64_t N, int64_t T) {
+    return syn_sparse_ws(B, Nin, N, T, false);
+}
+
 int syn_project_events(int64_t B, int64_t Nin, int64_t N, int64_t T, const float *W_t, const uint32_t *S_in,
                        const float *bias, float *I, void *stream) {
+    return syn_project_events_ws(B, Nin, N, T, W_t, S_in, bias, I, nullptr, 0, stream);
+}
+
+int syn_project_events_ws(int64_t B, int64_t Nin, int64_t N, int64_t T, const float *W_t, const uint32_t *S_in,
+                          const float *bias, float *I, void *workspace, size_t workspace_bytes, void *stream) {
     if (B < 0 || Nin < 0 || N < 0 || T < 0) return fail(ALIF_ESHAPE, "negative size");
     if (B == 0 || N == 0 || T == 0) return ALIF_OK;
-    if (Nin == 0) {  // no inputs: I = bias
-        return launch_status(launch_syn_project_events(B, 0, N, T, W_t, S_in, bias, I,
-                                                       static_cast<cudaStream_t>(stream)),
-                             "syn_project_events");
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const uint32_t *dense = nullptr;
+    if (Nin > 0) {  // without inputs I = bias
+        if (!W_t || !S_in || !I) return fail(ALIF_EINVAL, "NULL pointer");
+        if (((Nin + 1023) / 1024) * 1024 * N >= (1LL << 31))
+            return fail(ALIF_EUNSUPPORTED, "syn_project_events needs ceil(Nin/1024)*1024*N < 2^31");
+        const size_t need = workspace ? syn_sparse_ws(B, Nin, N, T, false) : 0;
+        if (need) {
+            if (!aligned(workspace, 256)) return fail(ALIF_ESHAPE, "workspace must be 256-byte aligned");
+            if (workspace_bytes < need) return fail(ALIF_EWORKSPACE, "workspace too small: need %zu bytes", need);
+            const int e = launch_syn_sparse(B, Nin, N, T, W_t, nullptr, nullptr, 0, S_in, bias, I, workspace, &dense, st);
+            if (e) return launch_status(e, "syn_project_events sparse launch");
+        }
     }
-    if (!W_t || !S_in || !I) return fail(ALIF_EINVAL, "NULL pointer");
-    if (((Nin + 1023) / 1024) * 1024 * N >= (1LL << 31))
-        return fail(ALIF_EUNSUPPORTED, "syn_project_events needs ceil(Nin/1024)*1024*N < 2^31");
-    return launch_status(launch_syn_project_events(B, Nin, N, T, W_t, S_in, bias, I, static_cast<cudaStream_t>(stream)),
-                         "syn_project_events");
+    return launch_status(launch_syn_project_events(B, Nin, N, T, W_t, S_in, bias, I, dense, st), "syn_project_events");
 }
 
 }  // extern "C"

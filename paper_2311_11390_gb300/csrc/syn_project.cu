@@ -72,6 +72,7 @@ struct Args {
     float *I;
     int tiles_m, tiles_t, nk;
     long long tiles;
+    const uint32_t *dense;  // NULL or dense[1]: every tile; else dense[0] time tiles, listed from dense[64]
     int *status;
 };
 
@@ -91,6 +92,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     proj_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
                 const __grid_constant__ CUtensorMap tm_s, const Args A) {
     extern __shared__ unsigned char smem_raw[];
+    const uint32_t *dense = A.dense && !__ldg(A.dense + 1) ? A.dense + 64 : nullptr;
+    const long long tiles = dense ? (long long)__ldg(A.dense) * A.tiles_m : A.tiles;
+    if (blockIdx.x >= tiles) return;
     // 1024-byte aligned base for the swizzled tiles
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -140,7 +144,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int nk = A.nk;
     auto tile_coords = [&](long long tile, int &m0, long long &t0, long long &b) {
         const int mt = (int)(tile % A.tiles_m);
-        const long long rest = tile / A.tiles_m;
+        const long long at = tile / A.tiles_m, rest = dense ? (long long)__ldg(dense + at) : at;
         m0 = mt * BM;
         t0 = (rest % A.tiles_t) * BN;
         b = rest / A.tiles_t;
@@ -155,7 +159,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ---- loads: spike words, then the weight slab, NA slabs ahead of the MMAs
         if (lane == 0) {
             long long &g = tma_issued;
-            for (long long tile = blockIdx.x; tile < A.tiles && !*abort_flag; tile += gridDim.x) {
+            for (long long tile = blockIdx.x; tile < tiles && !*abort_flag; tile += gridDim.x) {
                 int m0;
                 long long t0, b;
                 tile_coords(tile, m0, t0, b);
@@ -183,7 +187,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ---- tensor core: 8 MMAs per slab into the tile's accumulator
         if (lane == 0) {
             long long g = 0, it = 0;
-            for (long long tile = blockIdx.x; tile < A.tiles && !*abort_flag; tile += gridDim.x, ++it) {
+            for (long long tile = blockIdx.x; tile < tiles && !*abort_flag; tile += gridDim.x, ++it) {
                 const int buf = (int)(it & 1);
                 const uint32_t dacc = tmem + (uint32_t)(buf * 256);
                 if (it >= 2 && !mbar_wait_bounded(&acc_free[buf], (uint32_t)(((it >> 1) - 1) & 1))) {
@@ -220,7 +224,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int bw = warp - EPI_WARPS;
         const int jh = bw >> 1, tb0 = 4 * (bw & 1);
         long long g = 0;
-        for (long long tile = blockIdx.x; tile < A.tiles && !*abort_flag; tile += gridDim.x) {
+        for (long long tile = blockIdx.x; tile < tiles && !*abort_flag; tile += gridDim.x) {
             int m0;
             long long t0, b;
             tile_coords(tile, m0, t0, b);
@@ -283,7 +287,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ---- epilogue warps: TMEM lanes 32 w .. 32 w + 31 = neuron rows of the tile
         long long it = 0;
         const bool vec = ((A.T & 3) == 0) && ((reinterpret_cast<uintptr_t>(A.I) & 15u) == 0);
-        for (long long tile = blockIdx.x; tile < A.tiles && !*abort_flag; tile += gridDim.x, ++it) {
+        for (long long tile = blockIdx.x; tile < tiles && !*abort_flag; tile += gridDim.x, ++it) {
             int m0;
             long long t0, b;
             tile_coords(tile, m0, t0, b);
@@ -429,10 +433,11 @@ int launch_split_pad(const float *W, long long N, long long Nin, long long ldw, 
     return (int)cudaGetLastError();
 }
 
+// dense: NULL, or the list of (batch element, 256-step) tiles to compute (launch_syn_sparse).
 // Returns 0, a CUDA error code (> 0), or -1/-2 when the tensor maps cannot be built.
 int launch_syn_project(long long B, long long Nin, long long N, long long T, const uint16_t *W_hi,
                        const uint16_t *W_lo, long long ldw, const uint32_t *S, const float *bias, float *I,
-                       int *status, cudaStream_t stream) {
+                       const uint32_t *dense, int *status, cudaStream_t stream) {
     using namespace proj;
     CUtensorMap mh, ml;
     int rc = make_map(&mh, W_hi, N, ldw);
@@ -452,6 +457,7 @@ int launch_syn_project(long long B, long long Nin, long long N, long long T, con
     A.tiles_m = (int)((N + BM - 1) / BM);
     A.tiles_t = (int)((T + BN - 1) / BN);
     A.nk = (int)((Nin + BK - 1) / BK);
+    A.dense = dense;
     A.status = status;
     const long long tiles = (long long)A.tiles_m * A.tiles_t * B;
     A.tiles = tiles;

@@ -95,6 +95,7 @@ struct Args {
     const uint32_t *S;
     const float *bias;
     float *I;
+    const uint32_t *dense;  // NULL or dense[1]: every chunk; else those of dense[0] tiles, listed from dense[64]
 };
 
 template <int NPT>
@@ -107,7 +108,10 @@ __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args
     int *pos = reinterpret_cast<int *>(smem + C::ACC_BYTES + (size_t)MAX_EVENTS * 2);  // [GROUPS][32] first slots
     int *off = pos + GROUPS * 32;                                                  // [33] first event of step t
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long units = A.B * A.nwords;
+    // units are chunks; with a list, a tile's eight in order (those past T are passed over)
+    const uint32_t *dense = A.dense && !__ldg(A.dense + 1) ? A.dense + 64 : nullptr;
+    const long long units = dense ? 8LL * __ldg(A.dense) : A.B * A.nwords;
+    const long long tiles_t = (A.nwords + 7) / 8;
     const int nblk = (int)((A.Nin + IN_BLOCK - 1) / IN_BLOCK);
     for (long long nb = 0; nb < A.N; nb += NB_BLOCK) {
         const long long i0 = nb + (long long)tid * NPT;  // this thread's first neuron
@@ -120,7 +124,13 @@ __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args
         }
         const bool any_live = live[0];
         for (long long u = blockIdx.x; u < units; u += gridDim.x) {
-            const long long b = u / A.nwords, c = u % A.nwords;
+            long long b = u / A.nwords, c = u % A.nwords;
+            if (dense) {
+                const long long tile = __ldg(dense + (u >> 3));
+                b = tile / tiles_t;
+                c = (tile - b * tiles_t) * 8 + (u & 7);
+                if (c >= A.nwords) continue;
+            }
             const int nt = (int)(A.T - c * 32 < 32 ? A.T - c * 32 : 32);  // steps in this chunk
 #pragma unroll
             for (int t = 0; t < 32; ++t)  // this thread's columns only
@@ -285,9 +295,9 @@ int launch_transpose_weights(const float *W, long long N, long long Nin, float *
 }
 
 int launch_syn_project_events(long long B, long long Nin, long long N, long long T, const float *Wt,
-                              const uint32_t *S, const float *bias, float *I, cudaStream_t st) {
+                              const uint32_t *S, const float *bias, float *I, const uint32_t *dense, cudaStream_t st) {
     using namespace pev;
-    Args A{B, Nin, N, T, (T + 31) / 32, Wt, S, bias, I};
+    Args A{B, Nin, N, T, (T + 31) / 32, Wt, S, bias, I, dense};
     const long long units = B * A.nwords;
     if (units == 0 || N == 0) return 0;
     static int sms = 0;

@@ -61,6 +61,22 @@ inline int make_rowmajor_map(CUtensorMap *map, const float *I, long long rows, l
     return r == CUDA_SUCCESS ? 0 : -2;
 }
 
+// FP32 currents as [B, N, T]; one box is 32 rows x 16 steps of one batch element (64-byte
+// swizzle), clipped at N and T.  Returns 0, -1 (no encoder) or -2 (rejected: I must be 16-byte
+// aligned and T a multiple of 4).
+inline int make_batch_rows_map(CUtensorMap *map, const float *I, long long B, long long N, long long T) {
+    auto enc = tensor_map_encoder();
+    if (!enc) return -1;
+    const cuuint64_t dims[3] = {(cuuint64_t)T, (cuuint64_t)N, (cuuint64_t)B};
+    const cuuint64_t strides[2] = {(cuuint64_t)T * 4, (cuuint64_t)T * 4 * (cuuint64_t)N};
+    const cuuint32_t box[3] = {16, 32, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float *>(I), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? 0 : -2;
+}
+
 // 2-D tiled TMA load global -> shared, completion on the mbarrier at `bar`.
 // The inner coordinate c0 times the element size must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_2d_u(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar) {
