@@ -63,6 +63,8 @@ def lib():
         "syn_project_ws": ([i64, i64, i64, i64, P, P, i64, P, P, P, P, sz, P], ctypes.c_int),
         "syn_project_backward_workspace_size": ([i64, i64, i64], sz),
         "syn_project_backward": ([i64, i64, i64, i64, P, P, P, P, P, P, P, sz, P], ctypes.c_int),
+        "syn_project_backward_lists_size": ([i64, i64, i64, i64], sz),
+        "syn_project_backward_ws": ([i64, i64, i64, i64, P, P, P, P, P, P, P, sz, P, sz, P], ctypes.c_int),
         "alif_unpack_spikes": ([i64, i64, P, P, P], ctypes.c_int),
         "alif_vanrossum_forward": ([i64, i64, P, P, f64, f64, i64, P, P, P], ctypes.c_int),
         "alif_pack_spikes": ([i64, i64, P, P, P], ctypes.c_int),
@@ -455,10 +457,13 @@ def syn_project_backward(S_words, grad_I, W=None, Nin=None, want_gW=True, want_g
     gW = torch.empty((N, Nin), dtype=torch.float32, device=dev) if want_gW else None
     gS = torch.empty((B, Nin, T), dtype=torch.float32, device=dev) if want_gS else None
     gb = torch.empty((N,), dtype=torch.float32, device=dev) if want_gb else None
-    wsz = int(lib().syn_project_backward_workspace_size(B, N, Nin))
+    L = lib()
+    wsz = int(L.syn_project_backward_workspace_size(B, N, Nin))
     ws = torch.empty(max(wsz, 4), dtype=torch.uint8, device=dev)
-    _check(lib().syn_project_backward(B, Nin, N, T, _ptr(W), _ptr(S_words), _ptr(grad_I), _ptr(gW), _ptr(gS),
-                                      _ptr(gb), _ptr(ws), wsz, _stream(dev)), "syn_project_backward")
+    lsz = int(L.syn_project_backward_lists_size(B, Nin, N, T)) if want_gW or want_gb else 0
+    lists = torch.empty(lsz, dtype=torch.uint8, device=dev) if lsz else None
+    _check(L.syn_project_backward_ws(B, Nin, N, T, _ptr(W), _ptr(S_words), _ptr(grad_I), _ptr(gW), _ptr(gS),
+                                     _ptr(gb), _ptr(ws), wsz, _ptr(lists), lsz, _stream(dev)), "syn_project_backward")
     return gW, gS, gb
 
 

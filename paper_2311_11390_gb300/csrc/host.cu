@@ -57,10 +57,11 @@ int launch_syn_sparse(long long B, long long Nin, long long N, long long T, cons
                       const uint16_t *lo, long long ldw, const uint32_t *S, const float *bias, float *I, void *work,
                       const uint32_t **dense, cudaStream_t st);
 
-size_t syn_project_backward_ws(long long B, long long N, long long Nin);
+size_t syn_project_backward_need(long long B, long long N, long long Nin);
 int launch_syn_project_backward(long long B, long long Nin, long long N, long long T, const float *W,
                                 const uint32_t *S, const float *gI, float *gW, float *gS, float *gb, void *ws,
-                                int *status, cudaStream_t stream);
+                                void *lists, int *status, cudaStream_t stream);
+size_t syn_grad_weights_ws(long long B, long long Nin, long long N, long long T);
 
 int launch_readout_forward(long long B, long long K, long long C, long long T, const uint32_t *S, const float *W,
                            const float *bias, const float *w, float w_sum, float *n, float *o, cudaStream_t st);
@@ -704,12 +705,23 @@ int syn_project_ws(int64_t B, int64_t Nin, int64_t N, int64_t T, const uint16_t 
 
 size_t syn_project_backward_workspace_size(int64_t B, int64_t N, int64_t Nin) {
     if (B <= 0 || N <= 0 || Nin < 0) return 0;
-    return syn_project_backward_ws(B, N, Nin);
+    return syn_project_backward_need(B, N, Nin);
 }
 
 int syn_project_backward(int64_t B, int64_t Nin, int64_t N, int64_t T, const float *W, const uint32_t *S_in,
                          const float *grad_I, float *grad_W, float *grad_Sin, float *grad_bias, void *workspace,
                          size_t workspace_bytes, void *stream) {
+    return syn_project_backward_ws(B, Nin, N, T, W, S_in, grad_I, grad_W, grad_Sin, grad_bias, workspace,
+                                   workspace_bytes, nullptr, 0, stream);
+}
+
+size_t syn_project_backward_lists_size(int64_t B, int64_t Nin, int64_t N, int64_t T) {
+    return syn_grad_weights_ws(B, Nin, N, T);
+}
+
+int syn_project_backward_ws(int64_t B, int64_t Nin, int64_t N, int64_t T, const float *W, const uint32_t *S_in,
+                            const float *grad_I, float *grad_W, float *grad_Sin, float *grad_bias, void *workspace,
+                            size_t workspace_bytes, void *lists, size_t lists_bytes, void *stream) {
     int rc = check_shape(B, N, T);
     if (rc) return rc;
     if (Nin < 0) return fail(ALIF_ESHAPE, "Nin < 0");
@@ -725,16 +737,22 @@ int syn_project_backward(int64_t B, int64_t Nin, int64_t N, int64_t T, const flo
     if (!grad_I) return fail(ALIF_EINVAL, "grad_I is required");
     if ((grad_W || grad_bias) && !S_in) return fail(ALIF_EINVAL, "S_in is required for grad_W / grad_bias");
     if (grad_Sin && !W) return fail(ALIF_EINVAL, "W is required for grad_Sin");
-    if ((grad_W || grad_bias || grad_Sin) && (!workspace || workspace_bytes < syn_project_backward_ws(B, N, Nin)))
-        return fail(ALIF_EWORKSPACE, "workspace too small: need %zu bytes", syn_project_backward_ws(B, N, Nin));
+    if ((grad_W || grad_bias || grad_Sin) && (!workspace || workspace_bytes < syn_project_backward_need(B, N, Nin)))
+        return fail(ALIF_EWORKSPACE, "workspace too small: need %zu bytes", syn_project_backward_need(B, N, Nin));
     if (!aligned(grad_I, 4) || (W && !aligned(W, 4)) || (grad_Sin && !aligned(grad_Sin, 4)) ||
         (S_in && !aligned(S_in, 4)) || !aligned(workspace, 256))
         return fail(ALIF_ESHAPE, "misaligned pointer (workspace needs 256 bytes, the rest 4)");
     Symbols *sy = nullptr;
     rc = symbols(&sy);
     if (rc) return rc;
+    if (lists) {
+        const size_t need = (grad_W || grad_bias) ? syn_grad_weights_ws(B, Nin, N, T) : 0;
+        if (!aligned(lists, 256)) return fail(ALIF_ESHAPE, "lists must be 256-byte aligned");
+        if (lists_bytes < need) return fail(ALIF_EWORKSPACE, "lists too small: need %zu bytes", need);
+        if (!need) lists = nullptr;
+    }
     const int r = launch_syn_project_backward(B, Nin, N, T, W, S_in, grad_I, grad_W, grad_Sin, grad_bias, workspace,
-                                              sy->status, st);
+                                              lists, sy->status, st);
     if (r < 0) return fail(ALIF_EUNSUPPORTED, "syn_project_backward: the driver cannot encode the tensor maps");
     return launch_status(r, "syn_project_backward launch");
 }

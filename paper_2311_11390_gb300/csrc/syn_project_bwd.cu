@@ -7,7 +7,8 @@
 // shared memory and each thread, owning one input, walks that input's spikes,
 // adding the staged g_I column of the 16 rows to its accumulators.  Per-(b, row)
 // partials go to a workspace and are summed over the batch in a fixed order
-// (deterministic).
+// (deterministic).  With a list workspace, sparse rasters take the kernels of syn_grad_weights.cu;
+// these then run only where the raster was too dense for the lists.
 // g_S is a dense product (W^T x g_I per batch element) on the tcgen05 tensor cores with both
 // operands split into two BF16 terms (syn_grad_input.cu).
 #include "common.cuh"
@@ -46,7 +47,8 @@ template <bool VG, bool VS>  // VG: g_I rows in 16-byte units (T % 4 == 0); VS: 
 __global__ void __launch_bounds__(LTHREADS, 1) gw_lane_kernel(const float *__restrict__ gI,
                                                               const uint32_t *__restrict__ S, long long N,
                                                               long long Nin, long long T, int nwin, int ldp,
-                                                              float *part, float *part_b) {
+                                                              float *part, float *part_b, const uint32_t *flags) {
+    if (flags && !__ldg(flags + 1)) return;  // the list path has computed everything
     extern __shared__ float sm[];
     float *gt = sm;                                                          // [LCH][LGS]
     uint32_t *wsl = reinterpret_cast<uint32_t *>(sm + (size_t)LCH * LGS);   // [2][LTHREADS][LCW] word slots
@@ -187,11 +189,13 @@ __global__ void __launch_bounds__(LTHREADS, 1) gw_lane_kernel(const float *__res
 
 // Fixed-order sum over the batch: g_W[i][j] = sum_b part[b][i][j]; g_bias[i] likewise.
 __global__ void gw_reduce_kernel(const float *part, const float *part_b, long long B, long long N, long long Nin,
-                                 int ldp, float *gW, float *gb) {
+                                 int ldp, float *gW, float *gb, const uint32_t *flags) {
+    if (flags && !__ldg(flags + 1)) return;
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < N * Nin) {
         const long long i = k / Nin, j = k % Nin;
         float s = 0.0f;
+#pragma unroll 8
         for (long long b = 0; b < B; ++b) s += part[(b * N + i) * ldp + j];
         if (gW) gW[k] = s;
     }
@@ -204,6 +208,8 @@ __global__ void gw_reduce_kernel(const float *part, const float *part_b, long lo
 
 }  // namespace pbwd
 
+int launch_syn_grad_weights(long long B, long long Nin, long long N, long long T, const uint32_t *S, const float *gI,
+                            float *gW, float *gb, void *work, const uint32_t **flags, cudaStream_t st);
 size_t syn_grad_input_ws(long long N, long long Nin);
 int launch_syn_grad_input(long long B, long long N, long long Nin, long long T, const float *W, const float *gI,
                           float *gS, void *ws, int *status, cudaStream_t stream);
@@ -215,15 +221,20 @@ static size_t gw_part_bytes(long long B, long long N, long long Nin) {
     return ((size_t)(B * N * ldp + B * N) * sizeof(float) + 255) & ~(size_t)255;
 }
 
-size_t syn_project_backward_ws(long long B, long long N, long long Nin) {
+size_t syn_project_backward_need(long long B, long long N, long long Nin) {
     return gw_part_bytes(B, N, Nin) + syn_grad_input_ws(N, Nin);
 }
 
 int launch_syn_project_backward(long long B, long long Nin, long long N, long long T, const float *W,
                                 const uint32_t *S, const float *gI, float *gW, float *gS, float *gb, void *ws,
-                                int *status, cudaStream_t stream) {
+                                void *lists, int *status, cudaStream_t stream) {
     using namespace pbwd;
     if ((gW || gb) && Nin > 0) {
+        const uint32_t *flags = nullptr;
+        if (lists) {
+            const int rc = launch_syn_grad_weights(B, Nin, N, T, S, gI, gW, gb, lists, &flags, stream);
+            if (rc) return rc;
+        }
         const int ldp = (int)((Nin + 3) & ~3LL);
         float *part = static_cast<float *>(ws);
         float *part_b = part + B * N * ldp;
@@ -245,11 +256,12 @@ int launch_syn_project_backward(long long B, long long Nin, long long N, long lo
         const dim3 grid((unsigned)((N + LR - 1) / LR), (unsigned)B, (unsigned)((Nin + LJ - 1) / LJ));
         long long aN = N, aNin = Nin, aT = T;
         int anwin = nwin, aldp = ldp;
-        void *args[] = {(void *)&gI, (void *)&S, &aN, &aNin, &aT, &anwin, &aldp, &part, &part_b};
+        void *args[] = {(void *)&gI, (void *)&S, &aN, &aNin, &aT, &anwin, &aldp, &part, &part_b, &flags};
         cudaError_t e = cudaLaunchKernel((const void *)kernel_for(vg, vs), grid, dim3(LTHREADS), args, LSMEM, stream);
         if (e != cudaSuccess) return (int)e;
         const long long total = N * Nin > N ? N * Nin : N;
-        gw_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(part, part_b, B, N, Nin, ldp, gW, gb);
+        gw_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, stream>>>(part, part_b, B, N, Nin, ldp, gW, gb,
+                                                                                 flags);
         e = cudaGetLastError();
         if (e != cudaSuccess) return (int)e;
     }

@@ -61,12 +61,12 @@ inline size_t layout(long long tiles, int rec, void *base, Work *w) {
     return at + (size_t)tiles * CHUNKS * rec;
 }
 
-// Starts the workspace: no dense tile yet, or all of them if a sample of the raster has more than
+// Starts a workspace's flags: [0] no dense tile yet, [1] whether a sample of the raster has more than
 // `limit` active inputs per step.  One block, 4 words per thread (131 000 input steps; 32 words took
 // 30 us: one SM's random reads).
 constexpr int SAMPLE = 4;
 __global__ void __launch_bounds__(1024, 1) sample_kernel(const uint32_t *__restrict__ S, long long words, long long Nin,
-                                                         float limit, const Work ws) {
+                                                         float limit, uint32_t *flags) {
     __shared__ int part[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long n = words < 1024 * SAMPLE ? words : 1024 * SAMPLE;
@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(1024, 1) sample_kernel(const uint32_t *__restr
     if (warp == 0) {
         c = __reduce_add_sync(FULL, part[lane]);
         if (lane == 0) {
-            ws.ndense[0] = 0u;
-            ws.ndense[1] = (float)c * (float)Nin > limit * 32.0f * (float)n;
+            flags[0] = 0u;
+            flags[1] = (float)c * (float)Nin > limit * 32.0f * (float)n;
         }
     }
 }
@@ -442,6 +442,12 @@ __global__ void __launch_bounds__(THREADS, 1) sums_kernel(const __grid_constant_
 
 }  // namespace sparse
 
+int launch_density_sample(const uint32_t *S, long long words, long long Nin, float limit, uint32_t *flags,
+                          cudaStream_t st) {
+    sparse::sample_kernel<<<1, 1024, 0, st>>>(S, words, Nin, limit, flags);
+    return (int)cudaGetLastError();
+}
+
 // Workspace bytes of the sparse projection; 0 where it is not used: more inputs than a weight tile
 // holds, or a product too small to pay for the lists and three more launches.
 //   * In place of the tensor cores: from 6e10 products on.  There (B = 16, 512 -> 1024, T = 8000) the
@@ -478,14 +484,13 @@ int launch_syn_sparse(long long B, long long Nin, long long N, long long T, cons
     // at 9 of 1000, 3.11 against 1.37 at 15 of 512), so there only the records' capacity counts.
     const float room = cap_of((int)Nin) / 32.0f, even = 0.0214f * Nin - 4.5f;
     const float limit = !hi || even > room ? room : even > 6.5f ? even : 6.5f;
-    sample_kernel<<<1, 1024, 0, st>>>(S, B * Nin * A.nch, Nin, limit, A.ws);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return (int)e;
+    const int rc = launch_density_sample(S, B * Nin * A.nch, Nin, limit, A.ws.ndense, st);
+    if (rc) return rc;
     CUtensorMap out = {};
     const bool tma = make_batch_rows_map(&out, I, B, N, T) == 0;
     const auto sums = hi ? (tma ? sums_kernel<true, true> : sums_kernel<true, false>)
                          : (tma ? sums_kernel<false, true> : sums_kernel<false, false>);
-    e = cudaFuncSetAttribute(sums, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    cudaError_t e = cudaFuncSetAttribute(sums, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return (int)e;
     int dev = 0, sms = 0;
     e = cudaGetDevice(&dev);
