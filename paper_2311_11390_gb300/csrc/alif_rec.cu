@@ -13,18 +13,25 @@
 //      all N neurons from the G CTAs' shared memory (distributed shared
 //      memory) -- at most one spike per neuron and Block, since the ARP
 //      (T_eff = max(T_R, 2) >= T_R) allows no second one -- and lists them;
-//   2. each thread adds W_rec[i][j] for every listed spike (j, t) into its
-//      column of a [T_R x neurons] double-single shared accumulator, started
-//      from the feedforward current I_ff[t] of its row (W_rec is stored
-//      transposed, so a warp reads 128 contiguous bytes per spike).  The
-//      weights of up to WCH spikes are copied into shared memory together
-//      (cp.async, one round trip), and the feedforward current of Block n+1
-//      is copied into a second accumulator while Block n is resolved, so
-//      neither HBM read sits on the Block's critical path;
-//   3. each thread steps its neuron through the Block (Eqs 1-5, state form)
-//      with the current, V and a in double-single, so that every spike
-//      decision is the one exact arithmetic takes (a flip needs a margin near
-//      1e-12); it publishes the step of its spike (or none) for the next Block.
+//   2. the weights W_rec[i][j] of the listed spikes are copied into shared memory together
+//      (cp.async, one round trip for up to WCH spikes; W_rec is stored transposed, so a warp reads
+//      128 contiguous bytes per spike) while the spikes are sorted by step; spikes beyond WCH are
+//      added into the Block's currents beforehand, WCH at a time;
+//   3. each thread steps its neuron through the Block (Eqs 1-5, state form): the total current of a
+//      step, I_ff plus the weights of the step's spikes, V and a in double-single, so that every
+//      spike decision is the one exact arithmetic takes (a flip needs a margin near 1e-12).  At most
+//      one spike falls into a Block, so the spike's effects and the rare margins that FP32 cannot
+//      decide stand under branches, and the spike word is written once per Block.  It publishes the
+//      step of its spike (or none) for the next Block.
+// The Block's currents are kept neuron-major, so that they move as 16-byte units (VW steps) between
+// global memory, shared memory and registers; those of Block n+1 are copied into a second buffer
+// while Block n is resolved.
+// What bounds it: the latency of each Block's chain (cluster barrier 1.7k cycles, gather and list 1.1k,
+// weights 2k, the sums of the weights 3k, the double-single steps 2.5k at N = 1024, T_R = 20 and 27
+// spikes a Block) with one or two warps per scheduler.  B = 32, N = 1024, T = 4000: 1.20 ms (1.97 ms with
+// a shared double-single accumulator per step, single-float copies and every step under its own
+// branches).  Helper warps for the sums and the stores: 1.45 ms, their instructions compete with the
+// steps'.
 // The total current I_ff + I_rec, rounded to FP32, is written out for the backward, with the
 // spike words, the checkpoints every ALIF_CKPT_STEPS steps and the final state
 // in the layouts of alif_forward.  Every CTA of a cluster runs the same number
@@ -42,13 +49,16 @@ namespace rec {
 constexpr int MAX_G = 8;           // portable cluster size
 constexpr int MAX_PER = 1024;      // neurons per CTA
 constexpr int NO_SPIKE = -1;
-constexpr int MAX_WCH = 32;        // recurrent weights copied together
+constexpr int MAX_WCH = 64;        // recurrent weights copied together
+constexpr uint32_t NO_STEP = 1023;  // step of the entries past the last spike (T_R <= 1023)
 
 struct Args {
     long long B, N, T, nwords, nckpt;
     int TR, G, per;
     int nbuf;  // 2: the next Block's current is prefetched into a second accumulator
     int wch;   // spikes whose weights are copied into shared memory together
+    int P;     // floats per neuron of a current buffer
+    int wide;  // 1: rows of W keep 16 bytes
     const float *Iff;
     const float *Wt;  // [N pre, N post]
     const AlifNeuron *nrn;
@@ -58,23 +68,43 @@ struct Args {
     AlifState *ckpt, *fin;
 };
 
-// acc [nbuf][TR][per + 1] (rows padded by one float, so that a warp reading or writing 32
-// rows' chunks through it spreads over the banks), acl [TR][per], wbuf [wch][per] (floats);
-// spk [2][per]; list [N]; wsum [64]
-__host__ __device__ constexpr size_t smem_bytes(int TR, int per, long long N, int nbuf, int wch) {
-    return (size_t)nbuf * TR * (per + 1) * 4 + (size_t)TR * per * 4 + (size_t)wch * per * 4 + (size_t)2 * per * 4 +
-           (size_t)N * 4 + 64 * 4;
+// Floats per neuron of a current buffer: an odd number of VW-float units, at least T_R, so that 32
+// neurons' units fall in distinct banks.
+constexpr int pitch_of(int TR, int VW) { return (((TR + VW - 1) / VW) | 1) * VW; }
+
+// cur [nbuf][per][P] currents, acl [per][P] their low parts where weights were added beforehand,
+// wbuf [wch][per] weights; spk [2][per]; list [N]; sorted [wch + 4]; wsum [32]
+inline size_t smem_bytes(const Args &A) {
+    return (size_t)(A.nbuf + 1) * A.per * A.P * 4 + (size_t)A.wch * A.per * 4 + (size_t)2 * A.per * 4 + (size_t)A.N * 4 +
+           (A.wch + 4) * 4 + 32 * 4;
 }
 
 // 4-byte asynchronous global -> shared copy (completion tracked by cp.async groups)
 __device__ __forceinline__ void cp_async4(float *dst, const float *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
+// the same for VW floats
+template <int VW>
+__device__ __forceinline__ void cp_async_vec(float *dst, const float *src) {
+    if constexpr (VW == 4)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+    else if constexpr (VW == 2)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+    else
+        cp_async4(dst, src);
+}
+template <int VW>
+struct alignas(4 * VW) Vec {
+    float v[VW];
+};
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // b v + x for double-single b, v, x: the product of the high parts split exactly (FMA), the
 // low-order terms added once (relative error about 2^-46); a shorter dependent chain than a
@@ -91,19 +121,20 @@ __device__ __forceinline__ df df_axpy(df b, df v, df x) {
 }
 
 // MAXT: the CTA size the register budget is sized for (256: up to 255 registers a thread, for
-// clusters of at most 256 neurons per CTA; 1024 otherwise)
-template <int MAXT>
-__global__ void __launch_bounds__(MAXT) rec_fwd_kernel(const Args A) {
+// clusters of at most 256 neurons per CTA; 1024 otherwise).  VW: floats per unit of the currents.
+template <int MAXT, int VW>
+__global__ void __launch_bounds__(MAXT, 1) rec_fwd_kernel(const Args A) {
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char smem[];
     const int per = A.per, TR = A.TR, G = A.G, nbuf = A.nbuf, wch = A.wch;
-    const int ld = per + 1;                                                          // acc row stride
-    float *acc = reinterpret_cast<float *>(smem);                                   // [nbuf][TR][ld] hi
-    float *acl = acc + (size_t)nbuf * TR * ld;                                       // [TR][per] lo
-    float *wbuf = acl + (size_t)TR * per;                                            // [wch][per] weights
+    const int P = A.P;
+    float *bufs = reinterpret_cast<float *>(smem);                                  // [nbuf][per][P]
+    float *acl = bufs + (size_t)nbuf * per * P;                                      // [per][P]
+    float *wbuf = acl + (size_t)per * P;                                             // [wch][per]
     int *spk = reinterpret_cast<int *>(wbuf + (size_t)wch * per);                    // [2][per]
     uint32_t *list = reinterpret_cast<uint32_t *>(spk + 2 * per);                    // [N] (j << 10) | t
-    int *wsum = reinterpret_cast<int *>(list + A.N);                                 // [32] + total
+    uint32_t *sorted = list + A.N;                                                   // (slot << 10) | t by step
+    int *wsum = reinterpret_cast<int *>(sorted + wch + 4);                           // [32] warps' counts
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = (per + 31) >> 5;
     const int rank = (int)cl.block_rank();
     const long long b = blockIdx.x / G;
@@ -114,64 +145,63 @@ __global__ void __launch_bounds__(MAXT) rec_fwd_kernel(const Args A) {
     AlifNeuron nr{};
     if (live) nr = A.nrn[i];
     const df beta{nr.beta_hi, nr.beta_lo}, p{nr.p_hi, nr.p_lo}, c{nr.c_hi, nr.c_lo};
+    const float d = nr.d, th0 = nr.theta0;
     df v{0.0f, 0.0f}, a{0.0f, 0.0f};
-    int rem = 0;
+    int adm = 0;  // first step of the Block that admits input (Eq 4)
     if (live && A.init) {
         const AlifState s = A.init[row];
-        rem = s.rem > 0 ? s.rem : 0;
-        v = df{rem > 0 ? 0.0f : s.v, 0.0f};
+        adm = s.rem > 0 ? s.rem : 0;
+        v = df{adm > 0 ? 0.0f : s.v, 0.0f};
         a = df{s.a, 0.0f};
     }
-    uint32_t word = 0;
+    uint32_t word = 0;  // the spike word that holds the next step, so far
+    uint32_t *spikes = A.spikes + row * A.nwords;
     const long long nb = (A.T + TR - 1) / TR;
-    // A warp moves its 32 rows' Block chunks (row-contiguous in global memory) with
-    // element e = 32 j + lane at row e / cm, step e % cm, so that each access touches a
-    // few sectors instead of 32 rows; r and t advance by the quotient and remainder of
-    // 32 / cm.
+    // A warp moves its 32 neurons' Block chunks (contiguous in global memory) unit by unit: unit
+    // e = 32 j + lane of the chunk is unit e % nu of neuron e / nu, the quotient and remainder advancing
+    // by those of 32 / nu.
     const long long wrow = (long long)rank * per + warp * 32;  // this warp's first neuron
     const int nrow = (int)(A.N - wrow < 32 ? A.N - wrow : 32);
     const long long grow0 = b * A.N + wrow;
-    // feedforward current of Block m into the warp's columns of its accumulator
-    auto load_ff = [&](long long m) {
-        const long long tb0 = m * TR;
-        const int cm = (int)(A.T - tb0 < TR ? A.T - tb0 : TR);
-        float *dst = acc + (size_t)(nbuf == 2 ? (int)(m & 1) : 0) * TR * ld + warp * 32;
-        const int q32 = 32 / cm, r32 = 32 - q32 * cm;
-        int r = lane / cm, t = lane - r * cm;
-        for (int e = lane; e < 32 * cm; e += 32) {
-            if (r < nrow) cp_async4(dst + (size_t)t * ld + r, A.Iff + (grow0 + r) * A.T + tb0 + t);
+    const int nu_full = TR / VW > 0 ? TR / VW : 1, q_full = 32 / nu_full, r_full = 32 - q_full * nu_full;
+    const int r0_full = lane / nu_full, u0_full = lane - r0_full * nu_full;
+    auto units = [&](int nu, auto move) {
+        int q32 = q_full, r32 = r_full, r = r0_full, u = u0_full;
+        if (nu != nu_full) {  // the last Block
+            q32 = 32 / nu;
+            r32 = 32 - q32 * nu;
+            r = lane / nu;
+            u = lane - r * nu;
+        }
+        for (int e = lane; e < 32 * nu; e += 32) {
+            if (r < nrow) move(r, u * VW);
             r += q32;
-            t += r32;
-            if (t >= cm) {
-                t -= cm;
+            u += r32;
+            if (u >= nu) {
+                u -= nu;
                 ++r;
             }
         }
     };
-    // the Block's FP32 total current (left in cur by the steps) out to I_total, same mapping
-    auto store_I = [&](const float *cur, long long tb0, int cm) {
-        const int q32 = 32 / cm, r32 = 32 - q32 * cm;
-        int r = lane / cm, t = lane - r * cm;
-        for (int e = lane; e < 32 * cm; e += 32) {
-            if (r < nrow) A.Iout[(grow0 + r) * A.T + tb0 + t] = cur[(size_t)t * ld + warp * 32 + r];
-            r += q32;
-            t += r32;
-            if (t >= cm) {
-                t -= cm;
-                ++r;
-            }
-        }
+    auto steps_of = [&](long long m) { return (int)(A.T - m * TR < TR ? A.T - m * TR : TR); };
+    auto buffer = [&](long long m) { return bufs + (size_t)(nbuf == 2 ? (int)(m & 1) : 0) * per * P; };
+    auto load_ff = [&](long long m) {  // feedforward current of Block m (cp.async)
+        float *dst = buffer(m) + warp * 32 * P;
+        const float *src = A.Iff + grow0 * A.T + m * TR;
+        units(steps_of(m) / VW, [&](int r, int t) { cp_async_vec<VW>(dst + r * P + t, src + (long long)r * A.T + t); });
     };
-    for (int t = 0; t < TR; ++t) acl[(size_t)t * per + tid] = 0.0f;
+    for (int t = 0; t < P; ++t) acl[tid * P + t] = 0.0f;
+    const int wk = tid / (per / 4), wcol4 = 4 * (tid - wk * (per / 4));  // this thread's part of the weight copies
+    const long long wq = (long long)rank * per + wcol4;
     load_ff(0);
     cp_async_commit();
     for (long long n = 0; n < nb; ++n) {
         const long long t0 = n * TR;
-        const int cnt = (int)(A.T - t0 < TR ? A.T - t0 : TR);
+        const int cnt = steps_of(n);
         // ---- 1. spikes of Block n-1 from every CTA of the cluster, listed as (j, t)
         int total = 0;
         if (n > 0) {
-            cl.sync();  // every CTA has published spk[(n-1) & 1]
+            cluster_wait();  // every CTA has published spk[(n-1) & 1]
             const int par = (int)((n - 1) & 1);
             int ts[MAX_G];
             int mine = 0;
@@ -192,134 +222,225 @@ __global__ void __launch_bounds__(MAXT) rec_fwd_kernel(const Args A) {
             }
             if (lane == 31) wsum[warp] = incl;
             __syncthreads();
-            if (warp == 0) {
-                const int wv = lane < nwarps ? wsum[lane] : 0;
-                int wi = wv;
+            int upto = lane < nwarps ? wsum[lane] : 0;  // spikes of the warps up to this lane's
 #pragma unroll
-                for (int l = 1; l < 32; l <<= 1) {
-                    const int up = __shfl_up_sync(FULL, wi, l);
-                    if (lane >= l) wi += up;
-                }
-                if (lane < nwarps) wsum[lane] = wi - wv;  // exclusive warp offsets
-                if (lane == 31) wsum[32] = wi;
+            for (int l = 1; l < 32; l <<= 1) {
+                const int up = __shfl_up_sync(FULL, upto, l);
+                if (lane >= l) upto += up;
             }
-            __syncthreads();
-            int pos = wsum[warp] + incl - mine;
+            total = __shfl_sync(FULL, upto, 31);
+            const int before = warp ? __shfl_sync(FULL, upto, warp - 1) : 0;
+            int pos = before + incl - mine;
 #pragma unroll
             for (int r = 0; r < MAX_G; ++r)
                 if (ts[r] != NO_SPIKE) list[pos++] = ((uint32_t)(r * per + tid) << 10) | (uint32_t)ts[r];
-            total = wsum[32];
             __syncthreads();
         }
-        // ---- 2. feedforward current plus the recurrent current, column tid of cur.
-        // cp.async groups complete in commit order: the weights of the first chunk are
-        // committed before the next Block's current, so waiting for all but the newest
-        // group leaves only that prefetch in flight.  The loop's trip count is the same
-        // in every thread (total is the CTA's), so every lane reaches each __syncwarp.
-        float *cur = acc + (size_t)(nbuf == 2 ? (int)(n & 1) : 0) * TR * ld;
+        float *cur = buffer(n);
         if (nbuf == 1 && n > 0) {
             load_ff(n);
             cp_async_commit();
         }
-        {
-            const float *Wcol = A.Wt + i;
-            bool pref = nbuf == 2 && n + 1 < nb;
-            int e0 = 0;
-            do {
-                const int nch = total - e0 < wch ? total - e0 : wch;
-                if (live)
-                    for (int k = 0; k < nch; ++k)
-                        cp_async4(wbuf + (size_t)k * per + tid, Wcol + (long long)(list[e0 + k] >> 10) * A.N);
-                cp_async_commit();
-                if (pref) {
-                    load_ff(n + 1);
-                    cp_async_commit();
-                    cp_async_wait<1>();
-                    pref = false;
-                } else {
-                    cp_async_wait<0>();
+        // ---- 2. weights.  cp.async groups complete in commit order: waiting for all but the newest
+        // leaves only the next Block's current in flight.  total and nch are the CTA's.
+        auto copy_weights = [&](int e0, int nch) {
+            if (A.wide) {  // 16 bytes of four neurons each, four spikes at a time
+                if (wq < A.N)
+                    for (int k = wk; k < nch; k += 4)
+                        cp_async_vec<4>(wbuf + k * per + wcol4, A.Wt + (long long)(list[e0 + k] >> 10) * A.N + wq);
+            } else if (live) {
+#pragma unroll 4
+                for (int k = 0; k < nch; ++k)
+                    cp_async4(wbuf + k * per + tid, A.Wt + (long long)(list[e0 + k] >> 10) * A.N + i);
+            }
+            cp_async_commit();
+        };
+        int e0 = 0;
+        const bool multi = total > wch;
+        for (; total - e0 > wch; e0 += wch) {  // more spikes than weight slots: added into the buffers
+            copy_weights(e0, wch);
+            cp_async_wait<0>();
+            __syncthreads();
+            if (live)
+                for (int k = 0; k < wch; ++k) {
+                    const int at = tid * P + (int)(list[e0 + k] & 1023u);
+                    const df s2 = two_sum(cur[at], wbuf[(size_t)k * per + tid]);
+                    cur[at] = s2.hi;
+                    acl[at] += s2.lo;
                 }
-                __syncwarp();  // the warp's copies of this Block's current are visible to every lane
-                if (live)
-                    for (int k = 0; k < nch; ++k) {
-                        const int t = (int)(list[e0 + k] & 1023u);
-                        const df s2 = two_sum(cur[t * ld + tid], wbuf[(size_t)k * per + tid]);
-                        cur[t * ld + tid] = s2.hi;
-                        acl[t * per + tid] += s2.lo;
-                    }
-                e0 += nch;
-            } while (e0 < total);
+            __syncthreads();
         }
-        // ---- 3. the Block's steps (state form of Eqs 1-5).  The current of step t + 1 and its
-        // product with c do not depend on the state, so they are formed during step t (issue is
-        // in order: left inside step t + 1 they would lengthen its dependent chain).
+        const int nch = total - e0;
+        copy_weights(e0, nch);
+        const bool pref = nbuf == 2 && n + 1 < nb;
+        if (pref) {
+            load_ff(n + 1);
+            cp_async_commit();
+        }
+        for (int e = tid; e < nch; e += per) {  // by step, and within one in the order of the list
+            const uint32_t mine = (list[e0 + e] & 1023u) << 6 | (uint32_t)e;
+            int at = 0;
+#pragma unroll 8
+            for (int o = 0; o < nch; ++o) at += ((list[e0 + o] & 1023u) << 6 | (uint32_t)o) < mine;
+            sorted[at] = (uint32_t)e << 10 | mine >> 6;
+        }
+        if (tid < 4) sorted[nch + tid] = NO_STEP;
+        if (pref)
+            cp_async_wait<1>();
+        else
+            cp_async_wait<0>();
+        __syncthreads();
+        // ---- 3. the Block's steps, VW at a time
         int sp = NO_SPIKE;
         if (live) {
-            // total current of step u in double-single; its FP32 rounding is left in cur for
-            // the warp's store below, and acl is cleared for the next Block
-            auto take = [&](int u) {
-                const df I = quick_two_sum(cur[u * ld + tid], acl[u * per + tid]);
-                acl[u * per + tid] = 0.0f;
-                cur[u * ld + tid] = I.hi;
-                return df_mul(c, I);
-            };
-            df xn = cnt > 0 ? take(0) : df{0.0f, 0.0f};
-            for (int t = 0; t < cnt; ++t) {
-                const long long k = t0 + t;
-                const df x = xn;
-                if (t + 1 < cnt) xn = take(t + 1);
-                if (A.ckpt && (k & (ALIF_CKPT_STEPS - 1)) == 0) {
-                    AlifState s;
-                    s.v = v.hi;
-                    s.a = a.hi;
-                    s.rem = rem;
-                    A.ckpt[row * A.nckpt + k / ALIF_CKPT_STEPS] = s;
+            const float *wcol = wbuf + tid;
+            // event k's weight is w0, the next one's w1, ev2 the entry after
+            uint32_t ev0 = sorted[0], ev1 = sorted[1], ev2 = sorted[2];
+            float w0 = wcol[(ev0 >> 10) * per], w1 = wcol[(ev1 >> 10) * per];
+            const uint32_t *evp = sorted + 3;
+            const int tck = A.ckpt ? (int)((ALIF_CKPT_STEPS - (t0 & (ALIF_CKPT_STEPS - 1))) & (ALIF_CKPT_STEPS - 1)) : TR;
+            float *mycur = cur + tid * P, *mylo = acl + tid * P;
+            int ck = tck;  // next step of the Block whose entering state is a checkpoint
+            for (int u = 0; u < cnt; u += VW) {
+                Vec<VW> I = *reinterpret_cast<const Vec<VW> *>(mycur + u), lo{};
+                if (multi) {
+                    lo = *reinterpret_cast<const Vec<VW> *>(mylo + u);
+                    *reinterpret_cast<Vec<VW> *>(mylo + u) = Vec<VW>{};
                 }
-                const df V = df_axpy(beta, v, rem == 0 ? x : df{0.0f, 0.0f});  // Eq 2, 4
+#pragma unroll
+                for (int s = 0; s < VW; ++s)
+                    while ((int)(ev0 & 1023u) == u + s) {  // the same spikes in every thread of the CTA
+                        const df s2 = two_sum(I.v[s], w0);
+                        I.v[s] = s2.hi;
+                        lo.v[s] += s2.lo;
+                        ev0 = ev1;
+                        w0 = w1;
+                        ev1 = ev2;
+                        w1 = wcol[(ev1 >> 10) * per];
+                        ev2 = *evp++;  // at most the fourth entry past the last spike's
+                    }
+                df x[VW];  // c I m (Eqs 2, 4)
+#pragma unroll
+                for (int s = 0; s < VW; ++s) {
+                    const df It = quick_two_sum(I.v[s], lo.v[s]);
+                    I.v[s] = It.hi;  // the FP32 total current
+                    x[s] = df_mul(c, It);
+                    if (u + s < adm) x[s] = df{0.0f, 0.0f};
+                }
+                *reinterpret_cast<Vec<VW> *>(mycur + u) = I;
+                auto checkpoint = [&](int t, df v, df a) {
+                    AlifState st;
+                    st.v = v.hi;
+                    st.a = a.hi;
+                    st.rem = adm > t ? adm - t : 0;
+                    A.ckpt[row * A.nckpt + (t0 + t) / ALIF_CKPT_STEPS] = st;
+                };
                 // Eq 1 against theta = theta0 + d a (Eq 5).  The FP32 difference dz of V.hi and
                 // fl(theta0 + d a.hi) is within 2^-24 (|dz| + |V.hi| + |theta| + |d a.hi|) of the
-                // double-single margin, so outside 2^-21 (...) its sign is the margin's; nearer,
-                // the threshold is formed in double-single and compared exactly as before.
-                const float thf = fmaf(nr.d, a.hi, nr.theta0);
-                const float dz = V.hi - thf;
-                bool S;
-                if (fabsf(dz) > 0x1p-21f * (fabsf(V.hi) + fabsf(thf) + fabsf(nr.d * a.hi))) {
-                    S = dz > 0.0f;
-                } else {
-                    const df th = df_add(df{nr.theta0, 0.0f}, df_mul_f(a, nr.d));
-                    S = df_cmp(V, th) > 0;
+                // double-single margin, so outside 2^-21 (...) its sign is the margin's.
+                if (ck >= u + VW || ck < u) {
+                    // The unit's steps without a branch; a bit per step whose margin is not clearly
+                    // negative.  Those are decided in order: a spike ends the Block for its neuron
+                    // (T_eff >= T_R), the membrane is 0 from there on.
+                    df vs[VW], as[VW];  // V of the step, a entering it
+                    unsigned near = 0;
+                    df vf = v, af = a;
+#pragma unroll
+                    for (int s = 0; s < VW; ++s) {
+                        vf = df_axpy(beta, vf, x[s]);  // Eq 2, 4
+                        vs[s] = vf;
+                        as[s] = af;
+                        const float thf = fmaf(d, af.hi, th0);
+                        if (!(vf.hi - thf < -0x1p-21f * (fabsf(vf.hi) + fabsf(thf) + fabsf(d * af.hi)))) near |= 1u << s;
+                        af = df_mul(p, af);  // Eq 5
+                    }
+                    while (near) {
+                        const int s = __ffs(near) - 1;
+                        near &= near - 1u;
+                        df vt = vs[0], at = as[0];
+#pragma unroll
+                        for (int k = 1; k < VW; ++k)
+                            if (k == s) {
+                                vt = vs[k];
+                                at = as[k];
+                            }
+                        const float thf = fmaf(d, at.hi, th0);
+                        const float dz = vt.hi - thf;
+                        bool S = dz > 0.0f;
+                        if (!(fabsf(dz) > 0x1p-21f * (fabsf(vt.hi) + fabsf(thf) + fabsf(d * at.hi))))
+                            S = df_cmp(vt, df_add(df{th0, 0.0f}, df_mul_f(at, d))) > 0;
+                        if (S) {
+                            af = df_add(df_mul(p, at), df{1.0f, 0.0f});
+                            for (int k = s + 1; k < VW; ++k) af = df_mul(p, af);
+                            vf = df{0.0f, 0.0f};
+                            sp = u + s;
+                            adm = sp + nr.teff;
+                            break;
+                        }
+                    }
+                    v = vf;
+                    a = af;
+                    continue;
                 }
-                if (S) {
-                    v = df{0.0f, 0.0f};
-                    rem = nr.teff - 1;
-                    sp = t;
-                } else {
-                    v = V;
-                    rem = rem > 0 ? rem - 1 : 0;
-                }
-                a = df_mul(p, a);                       // Eq 5; adding an exact 0 would leave it unchanged
-                if (S) a = df_add(a, df{1.0f, 0.0f});
-                word |= (S ? 1u : 0u) << (k & 31);
-                if ((k & 31) == 31 || k == A.T - 1) {
-                    A.spikes[row * A.nwords + (k >> 5)] = word;
-                    word = 0;
+                // a unit with a checkpoint: step by step
+#pragma unroll 1
+                for (int s = 0; s < VW; ++s) {
+                    const int t = u + s;
+                    df xs = x[0];
+#pragma unroll
+                    for (int k = 1; k < VW; ++k)
+                        if (k == s) xs = x[k];
+                    if (t < adm) xs = df{0.0f, 0.0f};  // after a spike earlier in this unit
+                    if (t == ck) {
+                        checkpoint(t, v, a);
+                        ck += ALIF_CKPT_STEPS;
+                    }
+                    v = df_axpy(beta, v, xs);  // Eq 2, 4
+                    const float thf = fmaf(d, a.hi, th0);
+                    const float dz = v.hi - thf;
+                    bool S = dz > 0.0f;
+                    if (!(fabsf(dz) > 0x1p-21f * (fabsf(v.hi) + fabsf(thf) + fabsf(d * a.hi)))) {
+                        const df th = df_add(df{th0, 0.0f}, df_mul_f(a, d));
+                        S = df_cmp(v, th) > 0;
+                    }
+                    a = df_mul(p, a);  // Eq 5
+                    if (S) {
+                        a = df_add(a, df{1.0f, 0.0f});
+                        v = df{0.0f, 0.0f};
+                        adm = t + nr.teff;
+                        sp = t;
+                    }
                 }
             }
-        }
-        if (A.Iout) {
-            __syncwarp();
-            store_I(cur, t0, cnt);
+            adm = adm > cnt ? adm - cnt : 0;
+            // the spike words that the Block completes
+            const long long ks = t0 + sp;
+            for (long long w = t0 >> 5; w < (t0 + cnt) >> 5; ++w) {
+                spikes[w] = word | (sp != NO_SPIKE && (ks >> 5) == w ? 1u << (ks & 31) : 0u);
+                word = 0;
+            }
+            if (sp != NO_SPIKE && (ks >> 5) == (t0 + cnt) >> 5) word |= 1u << (ks & 31);
         }
         spk[(n & 1) * per + tid] = sp;
+        cluster_arrive();  // the current goes out while the others arrive
+        if (A.Iout) {
+            __syncwarp();
+            float *dst = A.Iout + grow0 * A.T + t0;
+            const float *src = cur + warp * 32 * P;
+            units(cnt / VW, [&](int r, int t) {
+                *reinterpret_cast<Vec<VW> *>(dst + (long long)r * A.T + t) = *reinterpret_cast<const Vec<VW> *>(src + r * P + t);
+            });
+        }
     }
+    if (live && (A.T & 31)) spikes[A.T >> 5] = word;
     if (live && A.fin) {
         AlifState s;
         s.v = v.hi;
         s.a = a.hi;
-        s.rem = rem;
+        s.rem = adm;
         A.fin[row] = s;
     }
-    cl.sync();  // no CTA leaves while another may still read its shared memory
+    cluster_wait();  // no CTA leaves while another may still read its shared memory
 }
 
 // Spike raster delayed by D steps: out bit t = in bit t - D (0 for t < D).
@@ -376,20 +497,32 @@ int launch_alif_forward_recurrent(long long B, long long N, long long T, int TR,
     if (e != cudaSuccess) return (int)e;
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return (int)e;
-    // largest configuration that fits: prefetch first, then as many weights per copy as possible
-    size_t smem = 0;
+    A.wide = N % 4 == 0 && reinterpret_cast<uintptr_t>(Wt) % 16 == 0;
+    // steps per unit of the currents: 16 or 8 bytes where rows and Blocks keep them
+    const uintptr_t pa = reinterpret_cast<uintptr_t>(Iff) | (Iout ? reinterpret_cast<uintptr_t>(Iout) : 0);
+    int vw = (T % 4 == 0 && TR % 4 == 0 && pa % 16 == 0) ? 4 : (T % 2 == 0 && TR % 2 == 0 && pa % 8 == 0) ? 2 : 1;
+    // The largest configuration that fits: both current buffers first, then as many weights per copy
+    // as possible; last, single steps in rows without padding.
     A.nbuf = 0;
-    for (int nbuf = 2; nbuf >= 1 && !A.nbuf; --nbuf)
-        for (int wch = MAX_WCH; wch >= 4; wch /= 2) {
-            smem = smem_bytes(TR, per, N, nbuf, wch);
-            if (smem <= (size_t)optin) {
-                A.nbuf = nbuf;
-                A.wch = wch;
-                break;
-            }
-        }
-    if (!A.nbuf) return -1;
-    auto kern = per <= 256 ? rec_fwd_kernel<256> : rec_fwd_kernel<MAX_PER>;
+    auto fits = [&](int v, int pitch, int nbuf, int wch) {
+        A.P = pitch;
+        A.wch = wch;
+        A.nbuf = nbuf;
+        if (smem_bytes(A) > (size_t)optin) A.nbuf = 0;
+        vw = v;
+        return A.nbuf != 0;
+    };
+    bool found = false;
+    for (int nbuf = 2; nbuf >= 1 && !found; --nbuf)
+        for (int wch = MAX_WCH; wch >= 4 && !found; wch /= 2) found = fits(vw, pitch_of(TR, vw), nbuf, wch);
+    if (!found && !fits(1, TR, 1, 4)) return -1;
+    const size_t smem = smem_bytes(A);
+    auto kern = per <= 256 ? (vw == 4   ? rec_fwd_kernel<256, 4>
+                              : vw == 2 ? rec_fwd_kernel<256, 2>
+                                        : rec_fwd_kernel<256, 1>)
+                           : (vw == 4   ? rec_fwd_kernel<MAX_PER, 4>
+                              : vw == 2 ? rec_fwd_kernel<MAX_PER, 2>
+                                        : rec_fwd_kernel<MAX_PER, 1>);
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return (int)e;
     cudaLaunchConfig_t cfg = {};
