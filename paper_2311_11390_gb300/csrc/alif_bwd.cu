@@ -15,9 +15,10 @@
 // recurrences as warp scans and accumulates the parameter gradients.  Windows
 // without spikes or refractory carry-in take a lean path (plain decayed scans);
 // the others use segmented scans whose factors are zero at the resets.
-// Inputs are staged by 2-D TMA boxes (rows of 16 floats, 64-byte swizzle) into
-// a per-warp ring, newest window first, when T is a multiple of 16; otherwise
-// lanes read global memory directly.  E = 8 (256-step windows, one checkpoint
+// Inputs are staged into a per-warp ring, newest window first, by 2-D TMA boxes
+// (rows of 16 floats, 64-byte swizzle) when T is a multiple of 16 and by 1-D bulk
+// copies when it is a multiple of 4; otherwise lanes read global memory directly
+// (ragged.cuh: why).  E = 8 (256-step windows, one checkpoint
 // stride) keeps the window's register arrays small enough for four CTAs of four
 // warps per SM: the kernel is bound by the latency of its scan chains, and the
 // warps hide it.  E = 16 (512-step windows, two CTAs per SM) serves calls whose
@@ -32,6 +33,7 @@
 
 #include "bwd_scan.cuh"
 #include "common.cuh"
+#include "ragged.cuh"
 #include "tmap.h"
 
 namespace alif {
@@ -90,7 +92,8 @@ constexpr int smem_bytes() {
            WARPS * 10 * 32 * 4 + 1024;
 }
 
-// LOAD: 1 = 2-D TMA ring, 0 = direct global loads; E steps per lane (Geo)
+// LOAD: 1 = 2-D TMA ring (T a multiple of 16, aligned arrays), 2 = ring of 1-D bulk copies (T a multiple
+// of 4, aligned arrays), 0 = direct global loads; E steps per lane (Geo)
 template <int LOAD, bool GV, bool GA, int SG, int E>
 __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
     bwd_kernel(const __grid_constant__ CUtensorMap tmI, const __grid_constant__ CUtensorMap tmS,
@@ -121,7 +124,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
     long long p_row = gw;
     int p_wi = (int)A.nwin - 1;
     unsigned issued = 0, consumed = 0;
-    if (LOAD == 1) {
+    if (LOAD != 0) {
         if (lane == 0) {
             for (int s = 0; s < NSTAGE; ++s) mbar_init(&bars[s], 1);
             fence_mbar_init();
@@ -132,13 +135,23 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
         while (p_row < A.rows && issued - consumed < (unsigned)NSTAGE) {
             if (lane == 0) {
                 const int st = issued % NSTAGE;
-                const uint32_t dst = smem_u32(ring + st * STAGE), bar = smem_u32(&bars[st]);
-                const int y = (int)((p_row * A.T + (long long)p_wi * WIN) >> 4);
-                mbar_arrive_expect_tx(&bars[st], NARR * BOX);
-                tma_load_2d_u(dst, &tmI, 0, y, bar);
-                tma_load_2d_u(dst + BOX, &tmS, 0, y, bar);
-                if (GV) tma_load_2d_u(dst + 2 * BOX, &tmV, 0, y, bar);
-                if (GA) tma_load_2d_u(dst + (GV ? 3 : 2) * BOX, &tmA, 0, y, bar);
+                const long long s = p_row * A.T + (long long)p_wi * WIN;
+                if constexpr (LOAD == 1) {
+                    const uint32_t dst = smem_u32(ring + st * STAGE), bar = smem_u32(&bars[st]);
+                    const int y = (int)(s >> 4);
+                    mbar_arrive_expect_tx(&bars[st], NARR * BOX);
+                    tma_load_2d_u(dst, &tmI, 0, y, bar);
+                    tma_load_2d_u(dst + BOX, &tmS, 0, y, bar);
+                    if (GV) tma_load_2d_u(dst + 2 * BOX, &tmV, 0, y, bar);
+                    if (GA) tma_load_2d_u(dst + (GV ? 3 : 2) * BOX, &tmA, 0, y, bar);
+                } else {
+                    float *dst = ring + st * STAGE;
+                    const long long left = A.T - (long long)p_wi * WIN;
+                    const int n = (int)(left < WIN ? left : WIN);
+                    mbar_arrive_expect_tx(&bars[st], 2u * 4u * n);
+                    bulk_g2s(dst, A.I + s, 4u * n, &bars[st]);
+                    bulk_g2s(dst + WIN, A.gS + s, 4u * n, &bars[st]);
+                }
             }
             ++issued;
             if (--p_wi < 0) {
@@ -147,15 +160,34 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
             }
         }
     };
-    if (LOAD == 1) issue();
+    if (LOAD != 0) issue();
+    static_assert(LOAD < 2 || (!GV && !GA), "the 1-D ring holds I and dL/dS");
 
     const int t0 = E * lane;
     // this lane's E floats in a stage: 16-byte chunks ch0 .. ch0 + E/4 - 1 of box row t0 / 16, under the
     // 64-byte swizzle of that row (a quarter warp's 16-byte reads fall in distinct bank groups)
     const int swz = ((t0 >> 4) >> 1) & 3, ch0 = (t0 & 15) >> 2, brow = 16 * (t0 >> 4);
     bool dead = false;
+    auto load_state = [&](long long row, int wi) {
+        AlifState st{0.0f, 0.0f, 0};
+        if (A.ckpt)
+            st = A.ckpt[row * A.nckpt + (long long)Geo<E>::CK * wi];
+        else if (A.init)
+            st = A.init[row];
+        return st;
+    };
+    auto load_word = [&](long long row, int wi) {
+        const long long widx = (long long)wi * (WIN / 32) + (t0 >> 5);
+        return widx < A.nwords ? __ldg(A.spikes + row * A.nwords + widx) : 0u;
+    };
+    AlifState cs_next = load_state(gw, (int)A.nwin - 1);
+    uint32_t wd_next = load_word(gw, (int)A.nwin - 1);
+    // A row's work beside its windows counts where rows are short (4 windows at T = 1000, whose
+    // instructions it nearly equalled): the decays by shared squarings, the sums by a halving exchange
+    // and the next row's entry loaded during this row's last window took 900 instructions off each
+    // row: 168 -> 152 us at 32768 rows of 1000 steps.
     for (long long r = gw; r < A.rows && !dead; r += nw) {
-        const AlifNeuron nr = A.nrn[r % A.N];
+        const AlifNeuron nr = A.nrn[row_neuron(r, A.rows, A.N)];
         const df beta{nr.beta_hi, nr.beta_lo}, p{nr.p_hi, nr.p_lo};
         const float bf = beta.hi, pf = p.hi, c = nr.c_hi, d = nr.d, th0 = nr.theta0;
         const int teff = nr.teff;
@@ -166,45 +198,33 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
         // to the window's first input.
         float Pa0, Pa4, b4f, p4f;
         {
-            {
-                const df b4 = df_pow(beta, H), pa = df_pow(p, t0), p4 = df_pow(p, H);
-                Pa0 = pa.hi;
-                Pa4 = df_mul(pa, p4).hi;
-                b4f = b4.hi;
-                p4f = p4.hi;
+            // by squarings, as df_pow would take each of them
+            df b = beta, q = p, pa{1.0f, 0.0f};
+#pragma unroll
+            for (int h = 1; h < H; h *= 2) {
+                b = df_mul(b, b);
+                q = df_mul(q, q);
             }
-            df b8 = df_pow(beta, E), p8 = df_pow(p, E);
+            b4f = b.hi;
+            p4f = q.hi;
+            const df p4 = q;
 #pragma unroll
             for (int l = 0; l < 5; ++l) {
-                Bb[l] = b8.hi;
-                Bp[l] = p8.hi;
-                b8 = df_mul(b8, b8);
-                p8 = df_mul(p8, p8);
+                b = df_mul(b, b);
+                q = df_mul(q, q);
+                Bb[l] = b.hi;
+                Bp[l] = q.hi;
+                const df m = df_mul(pa, q);
+                if ((lane >> l) & 1) pa = m;
             }
+            Pa0 = pa.hi;
+            Pa4 = df_mul(pa, p4).hi;
         }
-        const uint32_t *bits = A.spikes + r * A.nwords;
-
-        auto load_state = [&](int wi) {
-            AlifState st{0.0f, 0.0f, 0};
-            if (A.ckpt)
-                st = A.ckpt[r * A.nckpt + (long long)Geo<E>::CK * wi];
-            else if (A.init)
-                st = A.init[r];
-            return st;
-        };
-        auto load_word = [&](int wi) {
-            const long long widx = (long long)wi * (WIN / 32) + (t0 >> 5);
-            return widx < A.nwords ? __ldg(bits + widx) : 0u;
-        };
-        AlifState cs_next = load_state((int)A.nwin - 1);
-        uint32_t wd_next = load_word((int)A.nwin - 1);
 
         float gcV = A.gfin ? A.gfin[2 * r] : 0.0f;      // dL/d(final v)
         float gca = A.gfin ? A.gfin[2 * r + 1] : 0.0f;  // dL/d(final a)
         // parameter sums: FP32 partials per window, double-single every 4096 steps
         // sums q = 0..4: beta, p, theta0, d, R
-#pragma unroll
-        for (int q = 0; q < 10; ++q) accs[32 * q] = 0.0f;
         float r_th0 = 0.0f, r_d = 0.0f, r_beta = 0.0f, r_p = 0.0f, r_R = 0.0f;
 
         for (int wi = (int)A.nwin - 1; wi >= 0; --wi) {
@@ -213,17 +233,18 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
             const bool last_window = wi == (int)A.nwin - 1;
             float x[E], g[E];
             const float *stg = nullptr;  // this window's stage (released at the end of the window)
-            if (LOAD == 1) {
+            const long long s0 = r * A.T + w;  // the window's first element
+            if (LOAD != 0) {
                 const int st = consumed % NSTAGE;
                 if (!mbar_wait_bounded(&bars[st], (consumed / NSTAGE) & 1u)) {
                     report_timeout(A.status);
                     dead = true;
                     break;
                 }
-                stg = ring + st * STAGE + brow;
+                stg = ring + st * STAGE + (LOAD == 1 ? brow : t0);
 #pragma unroll
                 for (int q = 0; q < E / 4; ++q) {
-                    const int o = 4 * ((ch0 + q) ^ swz);
+                    const int o = LOAD == 1 ? 4 * ((ch0 + q) ^ swz) : 4 * q;
                     const float4 u = *reinterpret_cast<const float4 *>(stg + o);
                     const float4 v = *reinterpret_cast<const float4 *>(stg + WIN + o);
                     x[4 * q] = u.x; x[4 * q + 1] = u.y; x[4 * q + 2] = u.z; x[4 * q + 3] = u.w;
@@ -236,7 +257,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
                     issue();
                 }
             } else {
-                const long long o = r * A.T + w + t0;
+                const long long o = s0 + t0;
 #pragma unroll
                 for (int k = 0; k < E; ++k) {
                     const bool ok = t0 + k < cnt;
@@ -256,7 +277,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
             auto trace_grads = [&](float (&gv)[E], float (&gav)[E]) {
 #pragma unroll
                 for (int k = 0; k < E; ++k) gv[k] = gav[k] = 0.0f;
-                if (LOAD == 1) {
+                if constexpr (LOAD == 1) {
 #pragma unroll
                     for (int q = 0; q < E / 4; ++q) {
                         const int o = 4 * ((ch0 + q) ^ swz);
@@ -270,12 +291,8 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
                         }
                     }
                 } else {
-                    const long long o = r * A.T + w + t0;
-#pragma unroll
-                    for (int k = 0; k < E; ++k) {
-                        if (GV) gv[k] = __ldg(A.gV + o + k);
-                        if (GA) gav[k] = __ldg(A.ga + o + k);
-                    }
+                    if (GV) ragged::read_direct<E>(A.gV + s0, t0, cnt, gv);
+                    if (GA) ragged::read_direct<E>(A.ga + s0, t0, cnt, gav);
                 }
 #pragma unroll
                 for (int k = 0; k < E; ++k)
@@ -287,8 +304,11 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
             const AlifState cs = cs_next;
             const uint32_t wd = wd_next;
             if (wi > 0) {
-                cs_next = load_state(wi - 1);
-                wd_next = load_word(wi - 1);
+                cs_next = load_state(r, wi - 1);
+                wd_next = load_word(r, wi - 1);
+            } else if (r + nw < A.rows) {
+                cs_next = load_state(r + nw, (int)A.nwin - 1);
+                wd_next = load_word(r + nw, (int)A.nwin - 1);
             }
             const int rem = cs.rem > 0 ? cs.rem : 0;
             const float vin = rem > 0 ? 0.0f : cs.v;
@@ -363,7 +383,8 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
                         // the span.
                         float Ab[E];  // beta (1 - S[t-1])
 #pragma unroll
-                        for (int k = 0; k < E; ++k) Ab[k] = ((rs >> k) & 1u) ? 0.0f : bf;
+                        for (int k = 0; k < E; ++k)
+                            Ab[k] = (k > 0 ? (sb >> (k - 1)) & 1u : prevbit) ? 0.0f : bf;
                         // the two half lanes' maps (b parts from 0); a half lane's decay is beta^H without
                         // a reset inside it and 0 with one
                         // the window's first input carries beta vin (0 after a refractory carry-in)
@@ -377,18 +398,15 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
                         }
                         const float LA0 = (rs & LOM) ? 0.0f : b4f, LA1 = (rs & HIM) ? 0.0f : b4f;
                         float Lb = fmaf(LA1, Lb0, Lb1);
-                        int nr = rs == 0u;  // no reset inside this lane's span
+                        // lanes from the nearest lane at or below this one that holds a reset: the span of
+                        // 2^l lanes ending here is free of resets where that is at least 2^l (a flag
+                        // shuffled and combined at each level cost 16000-step rows 1305 -> 1250 us, with
+                        // the reverse scan's)
+                        const unsigned rl = __ballot_sync(FULL, rs != 0u) << (31 - lane);
+                        const int free = __clz(rl);
 #pragma unroll
-                        for (int l = 0; l < 5; ++l) {
-                            const int unr = __shfl_up_sync(FULL, nr, 1 << l);
-                            const float ub = __shfl_up_sync(FULL, Lb, 1 << l);
-                            if (lane >= (1 << l)) {
-                                Lb = fmaf(nr ? Bb[l] : 0.0f, ub, Lb);
-                                nr &= unr;
-                            }
-                        }
-                        float eb = __shfl_up_sync(FULL, Lb, 1);
-                        if (lane == 0) eb = 0.0f;
+                        for (int l = 0; l < 5; ++l) Lb = up_fma(Lb, free >= (1 << l) ? Bb[l] : 0.0f, 1u << l, Lb);
+                        const float eb = up_fma(Lb, 1.0f, 1u, 0.0f);  // 0 on lane 0
                         // V[t0-1] carried across lanes (the entering membrane included)
                         float v = eb;
                         const float v3 = fmaf(LA0, v, Lb0);  // V[t0+H-1] from the half-lane decay
@@ -485,15 +503,12 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
                     }
                     {
                         // reverse affine map of the lane's 8 steps (G_V[t0] = LF G_V[t0+8] + Le); as above,
-                        // the decays of spans of whole lanes are exact powers or 0.  Steps whose reverse
-                        // factor is 0: a spike, the window's last step and beyond (t0 + k >= cnt - 1), or
-                        // every step when beta is 0
-                        const int kt = min(max(cnt - 1 - t0, 0), E);
-                        unsigned zf = (sb | (FULLM & ~((1u << kt) - 1u))) & FULLM;
-                        if (bf == 0.0f) zf = FULLM;
+                        // the decays of spans of whole lanes are exact powers or 0.  The reverse factor is 0
+                        // at a spike; past the window's last step it meets zeros only (the injections there
+                        // are 0, and nothing flows into lane 31)
                         float Fr[E];  // the reverse factors
 #pragma unroll
-                        for (int k = 0; k < E; ++k) Fr[k] = ((zf >> k) & 1u) ? 0.0f : bf;
+                        for (int k = 0; k < E; ++k) Fr[k] = ((sb >> k) & 1u) ? 0.0f : bf;
                         // half lanes: G_V[t0+H] = LF1 G_V[t0+E] + Le1, G_V[t0] = LF0 G_V[t0+H] + Le0
                         float Le0 = 0.0f, Le1 = 0.0f;
 #pragma unroll
@@ -501,20 +516,15 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
                             Le0 = fmaf(Fr[k], Le0, e[k]);
                             Le1 = fmaf(Fr[H + k], Le1, e[H + k]);
                         }
-                        const float LF1 = (zf & HIM) ? 0.0f : b4f;
-                        float Le = fmaf((zf & LOM) ? 0.0f : b4f, Le1, Le0);
-                        int nr = zf == 0u;
+                        const float LF1 = (sb & HIM) ? 0.0f : b4f;
+                        float Le = fmaf((sb & LOM) ? 0.0f : b4f, Le1, Le0);
+                        const int free = __clz(__brev(spk >> lane));  // lanes up to the nearest spike's
 #pragma unroll
                         for (int l = 0; l < 5; ++l) {
-                            const int dnr = __shfl_down_sync(FULL, nr, 1 << l);
                             const float de = __shfl_down_sync(FULL, Le, 1 << l);
-                            if (lane + (1 << l) < 32) {
-                                Le = fmaf(nr ? Bb[l] : 0.0f, de, Le);
-                                nr &= dnr;
-                            }
+                            if (lane + (1 << l) < 32) Le = fmaf(free >= (1 << l) ? Bb[l] : 0.0f, de, Le);
                         }
-                        float gnext = __shfl_down_sync(FULL, Le, 1);  // G_V[t0+E]
-                        if (lane == 31) gnext = 0.0f;
+                        float gnext = down_fma(Le, 1.0f, 1u, 0.0f);  // G_V[t0+E] (0 on lane 31)
                         float g4 = fmaf(LF1, gnext, Le1);  // G_V[t0+H] from the half-lane decay
 #pragma unroll
                         for (int k = E - 1; k > H; --k) {
@@ -534,11 +544,16 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
 
                 // ---- dL/dI and the parameter sums (both paths; on the lean path mb is all ones, rs 0)
                 {
-                    const float Vprev_lane = SAMESTEP ? 0.0f : __shfl_up_sync(FULL, V[E - 1], 1);
+                    [[maybe_unused]] const float Vprev_lane = SAMESTEP ? 0.0f : __shfl_up_sync(FULL, V[E - 1], 1);
                     const float Ga_next_lane = __shfl_down_sync(FULL, f[0], 1);
                     if (A.gI && cw > 0) {
-                        float *go = A.gI + r * A.T + w + t0;
-                        if (LOAD == 1 && t0 + E <= cw) {
+                        [[maybe_unused]] float *go = A.gI + s0 + t0;
+                        if constexpr (LOAD == 0) {
+                            float y[E];
+#pragma unroll
+                            for (int k = 0; k < E; ++k) y[k] = ((mb >> k) & 1u) ? c * e[k] : 0.0f;
+                            ragged::store<E>(A.gI + s0, t0, cw, y);
+                        } else if (t0 + E <= cw) {
                             const float2 c2 = make_float2(c, c);
 #pragma unroll
                             for (int q = 0; q < E / 4; ++q) {
@@ -608,7 +623,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
                 window(std::true_type{});
             else
                 window(std::false_type{});
-            if (LOAD == 1 && (GV || GA)) {  // release the stage (trace gradients were read from it)
+            if (LOAD != 0 && (GV || GA)) {  // release the stage (trace gradients were read from it)
                 __syncwarp();
                 fence_proxy_async_smem();
                 ++consumed;
@@ -621,59 +636,69 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
             r_R += s_R;
             if ((wi & (Geo<E>::FOLD - 1)) == 0) {  // fold 4096 steps of FP32 partials into double-single
                 const float rq[5] = {r_beta, r_p, r_th0, r_d, r_R};
+                if (wi + Geo<E>::FOLD >= (int)A.nwin) {  // the row's first fold
 #pragma unroll
-                for (int q = 0; q < 5; ++q) {
-                    const df u = df_add(df{accs[32 * q], accs[32 * (5 + q)]}, df{rq[q], 0.0f});
-                    accs[32 * q] = u.hi;
-                    accs[32 * (5 + q)] = u.lo;
+                    for (int q = 0; q < 5; ++q) {
+                        accs[32 * q] = rq[q];
+                        accs[32 * (5 + q)] = 0.0f;
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 5; ++q) {
+                        const df u = df_add(df{accs[32 * q], accs[32 * (5 + q)]}, df{rq[q], 0.0f});
+                        accs[32 * q] = u.hi;
+                        accs[32 * (5 + q)] = u.lo;
+                    }
                 }
                 r_th0 = r_d = r_beta = r_p = r_R = 0.0f;
             }
         }
         if (dead) break;
-        // deterministic warp reduction of the parameter sums (double-single butterfly)
-        df acc[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) acc[q] = df{accs[32 * q], accs[32 * (5 + q)]};
-#pragma unroll
-        for (int q = 0; q < 5; ++q) {
-#pragma unroll
-            for (int off = 16; off; off >>= 1) {
-                const df o{__shfl_xor_sync(FULL, acc[q].hi, off), __shfl_xor_sync(FULL, acc[q].lo, off)};
-                acc[q] = df_add(acc[q], o);
-            }
+        // deterministic warp reduction of the parameter sums (double-single butterfly).  Each exchange
+        // also halves the sums a lane goes on with: bit 4 of the lane splits {0 1 2 | 3 4}, bit 3
+        // {0 1 | 2} and {3 4 | }, bit 2 the rest, so that 8 additions do the work of 25.
+        auto acc = [&](int q) { return df{accs[32 * q], accs[32 * (5 + q)]}; };
+        auto swap_add = [&](df keep, df give, int off) {
+            return df_add(keep, df{__shfl_xor_sync(FULL, give.hi, off), __shfl_xor_sync(FULL, give.lo, off)});
+        };
+        const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+        const df a0 = swap_add(acc(h4 ? 3 : 0), acc(h4 ? 0 : 3), 16);
+        const df a1 = swap_add(acc(h4 ? 4 : 1), acc(h4 ? 1 : 4), 16);
+        const df a2 = swap_add(acc(2), acc(2), 16);  // of use where bit 4 is 0
+        const df b0 = swap_add(h3 ? a2 : a0, h3 ? a0 : a2, 8);
+        const df b1 = swap_add(a1, a1, 8);  // of use where bit 3 is 0
+        df sum = swap_add(h2 ? b1 : b0, h2 ? b0 : b1, 4);
+        sum = swap_add(sum, sum, 2);
+        sum = swap_add(sum, sum, 1);
+        // lanes 0, 4, 8, 16 and 20 hold sums 0 to 4: per-row partials as (hi, lo) pairs, chained to the
+        // time constants.  The same-step beta sum carries a factor beta: dbeta/dtau / beta = DT / tau^2
+        // (rows with beta < 1/2 are rewritten by the follow-up kernel)
+        if ((lane & 3) == 0 && !(h3 && (h4 || h2))) {
+            const int q = h4 ? (h2 ? 4 : 3) : h3 ? 2 : (h2 ? 1 : 0);
+            const float kb = SAMESTEP ? (bf > 0.0f ? nr.dbeta_dtau / bf : 0.0f) : nr.dbeta_dtau;
+            if (q < 2) sum = df_mul_f(sum, q == 0 ? kb : nr.dp_dtau);
+            const int slot = q == 0   ? ALIF_G_TAU_MEM
+                             : q == 1 ? ALIF_G_TAU_ADAPT
+                             : q == 2 ? ALIF_G_THETA0
+                             : q == 3 ? ALIF_G_D
+                                      : ALIF_G_R;
+            float *o = A.part + r * (2 * ALIF_NUM_PARAM_GRADS) + 2 * slot;
+            o[0] = sum.hi;
+            o[1] = sum.lo;
         }
         if (lane == 0) {
-            // per-row partials as (hi, lo) pairs, chained to the time constants
-            // the same-step beta sum carries a factor beta: dbeta/dtau / beta = DT / tau^2 (rows with
-            // beta < 1/2 are rewritten by the follow-up kernel)
-            const float kb = SAMESTEP ? (bf > 0.0f ? nr.dbeta_dtau / bf : 0.0f) : nr.dbeta_dtau;
-            const df gtm = df_mul_f(acc[0], kb), gta = df_mul_f(acc[1], nr.dp_dtau);
-            float *o = A.part + r * (2 * ALIF_NUM_PARAM_GRADS);
-            o[2 * ALIF_G_TAU_MEM] = gtm.hi;
-            o[2 * ALIF_G_TAU_MEM + 1] = gtm.lo;
-            o[2 * ALIF_G_TAU_ADAPT] = gta.hi;
-            o[2 * ALIF_G_TAU_ADAPT + 1] = gta.lo;
-            o[2 * ALIF_G_THETA0] = acc[2].hi;
-            o[2 * ALIF_G_THETA0 + 1] = acc[2].lo;
-            o[2 * ALIF_G_D] = acc[3].hi;
-            o[2 * ALIF_G_D + 1] = acc[3].lo;
-            o[2 * ALIF_G_R] = acc[4].hi;
-            o[2 * ALIF_G_R + 1] = acc[4].lo;
             if (A.ginit) {
                 A.ginit[2 * r] = bf * gcV;
                 A.ginit[2 * r + 1] = gca;
             }
         }
     }
-    if (LOAD == 1) {
-        while (consumed < issued) {
-            if (!mbar_wait_bounded(&bars[consumed % NSTAGE], (consumed / NSTAGE) & 1u)) {
-                report_timeout(A.status);
-                break;
-            }
-            ++consumed;
+    while (LOAD != 0 && consumed < issued) {  // never leave a copy in flight into this CTA's shared memory
+        if (!mbar_wait_bounded(&bars[consumed % NSTAGE], (consumed / NSTAGE) & 1u)) {
+            report_timeout(A.status);
+            break;
         }
+        ++consumed;
     }
 }
 
@@ -720,7 +745,8 @@ static int dispatch_sel(int sel, bool wide, const CUtensorMap *m, const bwd::Arg
         case 4: return launch_variant<1, false, false, SG, 8>(m, A, stream);
         case 5: return launch_variant<1, false, true, SG, 8>(m, A, stream);
         case 6: return launch_variant<1, true, false, SG, 8>(m, A, stream);
-        default: return launch_variant<1, true, true, SG, 8>(m, A, stream);
+        case 7: return launch_variant<1, true, true, SG, 8>(m, A, stream);
+        default: return launch_variant<2, false, false, SG, 8>(m, A, stream);
     }
 }
 
@@ -762,7 +788,8 @@ int launch_alif_backward(long long B, long long N, long long T, const float *I,
                (!gI || a16(gI)) && (n16 + 32 < (1LL << 31));
     // 512-step windows when the rows leave warp slots empty (each row's chain of windows is then the
     // limit, and longer windows halve it), 256-step windows (four CTAs per SM) otherwise; the wide
-    // kernel serves the TMA path without trace gradients
+    // kernel serves the tiled staging without trace gradients (512-step windows of other rows measured 33.4
+    // -> 29.3 us at 777 x 3001 steps, but summed the parameter gradients with 1.5 times the error)
     bool wide = g_bwd_window == 512 || (g_bwd_window == 0 && A.rows <= 8LL * g_sm_count_bwd);
     wide = wide && tma && !gV && !ga;
     const unsigned win = wide ? Geo<16>::WIN : Geo<8>::WIN;
@@ -779,7 +806,9 @@ int launch_alif_backward(long long B, long long N, long long T, const float *I,
             A.nwin = (T + Geo<8>::WIN - 1) / Geo<8>::WIN;
         }
     }
-    const int sel = (tma ? 4 : 0) | (gV ? 2 : 0) | (ga ? 1 : 0);
+    // rows of 4-float granules without trace gradients: the 1-D ring (see ragged.cuh for both sides)
+    const bool lin = !tma && T % 4 == 0 && a16(I) && a16(gS) && (!gI || a16(gI)) && !gV && !ga;
+    const int sel = lin ? 8 : (tma ? 4 : 0) | (gV ? 2 : 0) | (ga ? 1 : 0);
     switch (surrogate) {
         case 1: return dispatch_sel<1>(sel, wide, m, A, stream);
         case 2: return dispatch_sel<2>(sel, wide, m, A, stream);

@@ -23,7 +23,8 @@
 // Input staging: when T is a multiple of 16 the current is viewed as rows of
 // 16 floats and each window (16 such rows) is one 2-D TMA box with 64-byte
 // swizzle, so that the lanes' 16-byte reads hit distinct bank groups;
-// otherwise lanes read global memory directly.
+// when it is a multiple of 4 a window is one 1-D bulk copy; otherwise lanes read
+// global memory directly (ragged.cuh: why).
 //
 // Exactness of the spike decisions: the FP32 margin M = V~ - theta comes with
 // an error bound G, and |M| <= G is re-decided in double-single arithmetic from
@@ -47,6 +48,7 @@
 
 #include "common.cuh"
 #include "exact_membrane.cuh"
+#include "ragged.cuh"
 #include "tmap.h"
 
 namespace alif {
@@ -220,14 +222,16 @@ __device__ __forceinline__ float vabsmax(const float (&v)[E]) {
     }
 }
 
-// LOAD: 1 = 2-D TMA ring, 0 = direct global loads, 2 = fused projection (I computed from the input
-// events and the FP32 weight row staged in the warp's ring area, then written out)
+// LOAD: 1 = 2-D TMA ring (T a multiple of 16, aligned arrays), 3 = ring of 1-D bulk copies (T a
+// multiple of 4, aligned arrays), 0 = direct global loads, 2 = fused projection (I computed from the
+// input events and the FP32 weight row staged in the warp's ring area, then written out)
 template <int LOAD, bool VTR, bool ATR, int E>
 __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
     fwd_kernel(const __grid_constant__ CUtensorMap tm, const Args A) {
     constexpr int WIN = Geo<E>::WIN, H = Geo<E>::H, CK = Geo<E>::CK, NSTAGE = Geo<E>::NSTAGE;
     constexpr int STAGE_BYTES = Geo<E>::STAGE_BYTES, PDN = Geo<E>::PDN, PD_BYTES = Geo<E>::PD_BYTES;
     constexpr int RT_FLOATS = Geo<E>::RT_FLOATS;
+    constexpr bool RING = LOAD == 1 || LOAD == 3;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     unsigned char *sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);  // swizzled stages: 1024-aligned
@@ -249,7 +253,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
     const int nwin = (int)A.nwin;
     const int lastcnt = (int)(A.T - (long long)(nwin - 1) * WIN);
     unsigned issued = 0, consumed = 0;
-    if (LOAD == 1) {
+    if (RING) {
         if (lane == 0) {
             for (int s = 0; s < NSTAGE; ++s) mbar_init(&bars[s], 1);
             fence_mbar_init();
@@ -260,9 +264,15 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
         while (p_row < A.rows && issued - consumed < (unsigned)NSTAGE) {
             if (lane == 0) {
                 const int st = issued % NSTAGE;
-                mbar_arrive_expect_tx(&bars[st], STAGE_BYTES);
-                tma_load_2d_u(smem_u32(ring + st * WIN), &tm, 0,
-                              (int)((p_row * A.T + (long long)p_wi * WIN) >> 4), smem_u32(&bars[st]));
+                const long long s = p_row * A.T + (long long)p_wi * WIN;
+                if constexpr (LOAD == 1) {
+                    mbar_arrive_expect_tx(&bars[st], STAGE_BYTES);
+                    tma_load_2d_u(smem_u32(ring + st * WIN), &tm, 0, (int)(s >> 4), smem_u32(&bars[st]));
+                } else {
+                    const int n = p_wi == nwin - 1 ? lastcnt : WIN;
+                    mbar_arrive_expect_tx(&bars[st], 4u * n);
+                    bulk_g2s(ring + st * WIN, A.I + s, 4u * n, &bars[st]);
+                }
             }
             ++issued;
             if (++p_wi == nwin) {
@@ -271,7 +281,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
             }
         }
     };
-    if (LOAD == 1) issue();
+    if (RING) issue();
 
     bool dead = false;
     unsigned n_exact = 0, n_exact_spk = 0, n_rows = 0;
@@ -281,7 +291,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
     const int swz = ((t0 >> 4) >> 1) & 3, ch0 = (t0 & 15) >> 2, brow = 16 * (t0 >> 4);
 
     for (long long r = gw; r < A.rows && !dead; r += nw) {
-        const AlifNeuron nr = A.nrn[r % A.N];
+        const AlifNeuron nr = A.nrn[row_neuron(r, A.rows, A.N)];
         const df beta{nr.beta_hi, nr.beta_lo}, p{nr.p_hi, nr.p_lo};
         const float *Irow = A.I + r * A.T;
         float bias_i = 0.0f;
@@ -295,23 +305,44 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
         const float bf = nr.beta_hi, pf = nr.p_hi, c = nr.c_hi;
 
         // Warp tables: p^j (j = 0..WIN) as double-single pairs; span decays.
+        // By squarings shared by all powers (the products df_pow would take each of them by): the
+        // row's entry is a serial chain, which short rows of few warps wait for.
         float Pw0;  // p^{t0}
+        df bw;      // beta^WIN
         {
-            df q = df_pow(p, t0);
-            Pw0 = q.hi;
+            df b = beta, q = p, bk{1.0f, 0.0f}, pa{1.0f, 0.0f}, pe{1.0f, 0.0f};  // beta^(lane+1), p^t0, p^(E-1)
+#pragma unroll
+            for (int h = 1; h < E; h *= 2) {
+                const df m = df_mul(bk, b);
+                if ((lane + 1) & h) bk = m;
+                pe = df_mul(pe, q);
+                b = df_mul(b, b);
+                q = df_mul(q, q);
+            }
+            float bl = 0.0f;
+#pragma unroll
+            for (int l = 0; l < 5; ++l) {  // b = beta^(E 2^l), q = p^(E 2^l)
+                if (lane == 8 + l) bl = b.hi;
+                const df m = df_mul(pa, q);
+                if ((lane >> l) & 1) pa = m;
+                b = df_mul(b, b);
+                q = df_mul(q, q);
+            }
+            bw = b;
+            Pw0 = pa.hi;
 #pragma unroll
             for (int k = 0; k < E; ++k) {
-                pdh[t0 + k] = q.hi;
-                pdl[t0 + k] = q.lo;
-                q = df_mul(q, p);
+                pdh[t0 + k] = pa.hi;
+                pdl[t0 + k] = pa.lo;
+                pa = df_mul(pa, p);
             }
             if (lane == 31) {
-                pdh[WIN] = q.hi;
-                pdl[WIN] = q.lo;
+                pdh[WIN] = pa.hi;
+                pdl[WIN] = pa.lo;
             }
-            if (lane < H) rt[lane] = df_pow(beta, lane + 1).hi;
-            else if (lane >= 8 && lane < 13) rt[lane] = df_pow(beta, (long long)E << (lane - 8)).hi;
-            else if (lane == 13) rt[13] = df_pow(p, E - 1).hi;
+            if (lane < H) rt[lane] = bk.hi;
+            else if (lane >= 8 && lane < 13) rt[lane] = bl;
+            else if (lane == 13) rt[13] = pe.hi;
         }
         __syncwarp();
         const float2 *Bk2 = reinterpret_cast<const float2 *>(rt);  // (beta, beta^2), (beta^3, beta^4), ...
@@ -324,7 +355,6 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
         constexpr float us = 5.9604645e-8f * 1.015625f;
         float gC;
         {
-            const df bw = df_pow(beta, WIN);
             const float om = (1.0f - bw.hi) - bw.lo;
             gC = (E + 16.0f) * us * fminf(bw.hi / fmaxf(om, 0x1p-20f), 0x1p20f);
         }
@@ -353,17 +383,19 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
             const bool last = wi == nwin - 1;
             const int cnt = last ? lastcnt : WIN;
             float cx[E];
-            if (LOAD == 1) {
+            if (RING) {
                 const int st = consumed % NSTAGE;
                 if (!mbar_wait_bounded(&bars[st], (consumed / NSTAGE) & 1u)) {
                     report_timeout(A.status);
                     dead = true;
                     break;
                 }
-                const float *row16 = ring + st * WIN + brow;  // the box row holding this lane's steps
+                // LOAD 1: the box row holding this lane's steps
+                const float *row = ring + st * WIN + (LOAD == 1 ? brow : t0);
 #pragma unroll
                 for (int q = 0; q < E / 4; ++q) {
-                    const float4 u = *reinterpret_cast<const float4 *>(row16 + 4 * ((ch0 + q) ^ swz));
+                    const int o = LOAD == 1 ? 4 * ((ch0 + q) ^ swz) : 4 * q;
+                    const float4 u = *reinterpret_cast<const float4 *>(row + o);
                     cx[4 * q] = u.x; cx[4 * q + 1] = u.y; cx[4 * q + 2] = u.z; cx[4 * q + 3] = u.w;
                 }
                 __syncwarp();
@@ -412,8 +444,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
                 }
                 __syncwarp();  // the window's currents are visible to the warp's exact re-reads
             } else {
-#pragma unroll
-                for (int k = 0; k < E; ++k) cx[k] = (t0 + k < cnt) ? __ldg(Irow + w + t0 + k) : 0.0f;
+                ragged::read_direct<E>(Irow + w, t0, cnt, cx);
             }
             if (last) {
 #pragma unroll
@@ -618,7 +649,10 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
             if (VTR || ATR) {
                 float *vo = VTR ? A.vtr + r * A.T + w + t0 : nullptr;
                 float *ao = ATR ? A.atr + r * A.T + w + t0 : nullptr;
-                if (LOAD == 1 && t0 + E <= cnt) {
+                if constexpr (LOAD == 0) {
+                    if (VTR) ragged::store<E>(A.vtr + r * A.T + w, t0, cnt, vt);
+                    if (ATR) ragged::store<E>(A.atr + r * A.T + w, t0, cnt, a_el);
+                } else if (t0 + E <= cnt) {
 #pragma unroll
                     for (int q = 0; q < E / 4; ++q) {
                         if (VTR)
@@ -671,7 +705,7 @@ __global__ void __launch_bounds__(WARPS * 32, Geo<E>::MIN_BLOCKS)
         __syncwarp();  // the p^j table is rewritten for the next row
     }
 
-    if (LOAD == 1) {  // never leave a copy in flight into this CTA's shared memory
+    if (RING) {  // never leave a copy in flight into this CTA's shared memory
         while (consumed < issued) {
             const int st = consumed % NSTAGE;
             if (!mbar_wait_bounded(&bars[st], (consumed / NSTAGE) & 1u)) {
@@ -897,7 +931,7 @@ int launch_alif_forward(long long B, long long N, long long T, const float *I,
                (A.rows * T / 16 + 32 < (1LL << 31));
     // 512-step windows when the rows leave warp slots empty (each row's chain of windows is then
     // the limit, and longer windows halve it), 256-step windows (four CTAs per SM) otherwise; the
-    // wide kernel serves the TMA path without traces
+    // wide kernel serves the tiled staging without traces
     bool wide = g_fwd_window == 512 || (g_fwd_window == 0 && A.rows <= 8LL * g_sm_count);
     wide = wide && tma && !vtr && !atr;
     const long long win = wide ? Geo<16>::WIN : Geo<8>::WIN;
@@ -908,7 +942,9 @@ int launch_alif_forward(long long B, long long N, long long T, const float *I,
     }
     A.nwin = (T + (wide ? Geo<16>::WIN : Geo<8>::WIN) - 1) / (wide ? Geo<16>::WIN : Geo<8>::WIN);
     if (wide) return launch_fwd<1, false, false, 16>(tm, A, stream);
-    switch ((tma ? 4 : 0) | (vtr ? 2 : 0) | (atr ? 1 : 0)) {
+    // rows of 4-float granules: the 1-D ring (see ragged.cuh for both sides)
+    const bool lin = !tma && T % 4 == 0 && aligned16(I) && (!vtr || aligned16(vtr)) && (!atr || aligned16(atr));
+    switch ((lin ? 8 : tma ? 4 : 0) | (vtr ? 2 : 0) | (atr ? 1 : 0)) {
         case 0: return launch_fwd<0, false, false, 8>(tm, A, stream);
         case 1: return launch_fwd<0, false, true, 8>(tm, A, stream);
         case 2: return launch_fwd<0, true, false, 8>(tm, A, stream);
@@ -916,7 +952,11 @@ int launch_alif_forward(long long B, long long N, long long T, const float *I,
         case 4: return launch_fwd<1, false, false, 8>(tm, A, stream);
         case 5: return launch_fwd<1, false, true, 8>(tm, A, stream);
         case 6: return launch_fwd<1, true, false, 8>(tm, A, stream);
-        default: return launch_fwd<1, true, true, 8>(tm, A, stream);
+        case 7: return launch_fwd<1, true, true, 8>(tm, A, stream);
+        case 8: return launch_fwd<3, false, false, 8>(tm, A, stream);
+        case 9: return launch_fwd<3, false, true, 8>(tm, A, stream);
+        case 10: return launch_fwd<3, true, false, 8>(tm, A, stream);
+        default: return launch_fwd<3, true, true, 8>(tm, A, stream);
     }
 }
 

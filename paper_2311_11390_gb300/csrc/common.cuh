@@ -172,6 +172,11 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     }
 }
 
+// Neuron of row r of `rows` (B x N rows, N neurons); the 64-bit remainder costs some hundred cycles.
+__device__ __forceinline__ long long row_neuron(long long r, long long rows, long long N) {
+    return rows <= 0x7fffffffLL ? (long long)((unsigned)r % (unsigned)N) : r % N;
+}
+
 // 1-D bulk copy global -> shared, completion signalled on `bar` (tx bytes).
 // dst, src and bytes must be multiples of 16.
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
