@@ -56,12 +56,13 @@ class ALIFFunction(torch.autograd.Function):
                           for t in (tau_mem, tau_adapt, theta0, d, R)]
         words = out["spikes"]
         ctx.mark_non_differentiable(words)
+        ctx.set_materialize_grads(False)  # else the words receive a zero gradient, filled on every backward
         return S, words
 
     @staticmethod
     def backward(ctx, grad_S, _grad_words=None):
         I, spikes, ckpt, table = ctx.saved_tensors
-        grad_S = grad_S.contiguous().to(torch.float32)
+        grad_S = torch.zeros_like(I) if grad_S is None else grad_S.contiguous().to(torch.float32)
         gI, _, gp = alif.backward(I, table, spikes, grad_S, ckpt=ckpt, slope=ctx.slope,
                                   want_gI=ctx.needs_input_grad[0], surrogate=ctx.surrogate,
                                   attached=ctx.attached)

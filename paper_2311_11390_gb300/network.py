@@ -50,9 +50,10 @@ class Readout(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, S, W, bias, words, T, w_t, w_sum):
-        logits, counts = alif.readout_forward(words, T, W.detach().contiguous(),
+        Wd = W.detach().contiguous()
+        logits, counts = alif.readout_forward(words, T, Wd,
                                               None if bias is None else bias.detach().contiguous(), w_t, w_sum)
-        ctx.save_for_backward(W.detach().contiguous(), counts, w_t)
+        ctx.save_for_backward(Wd, counts, w_t)
         ctx.T, ctx.w_sum, ctx.has_bias = T, w_sum, bias is not None
         return logits
 
