@@ -14,9 +14,10 @@
 //   4. the state entering the next Block (Props 4 and 5): after a spike at k the membrane is 0,
 //      the rest of the Block lies in the refractory span (K <= T_R) and a = p^{K-1-k} (p a_k + 1);
 //      otherwise v = V~[K-1] and a = p^K a_in.
-// A warp holds 32 consecutive rows.  K = 16 when every row of the warp has T_eff >= 16, else 8, 4
-// or 2 (T_eff >= 2 always).  The state chain of a row costs O(1) dependent operations per Block, the
-// sequential depth of the method; the L chains run ahead of it.
+// A warp holds 32 consecutive rows.  K = 16 when every row of the warp has T_eff >= 16, else 8 or 4.
+// The state chain of a row costs O(1) dependent operations per Block, the sequential depth of the
+// method; the L chains run ahead of it.  Below T_eff = 4 a Block would be two steps, most of whose
+// work is per Block: those rows go step by step (group_steps).
 //
 // Input: stages of [32 rows x 64 steps] (two 2-D TMA boxes of 32 x 32 floats, 128-byte swizzle)
 // in a three-deep ring per warp; a lane reads its own row's K steps with 16-byte loads, which
@@ -89,8 +90,7 @@ __device__ __forceinline__ float max3f(float a, float b, float c) {
 
 template <int K>
 __device__ __forceinline__ float vmaxk(const float (&v)[K]) {
-    if constexpr (K == 2) return fmaxf(v[0], v[1]);
-    else if constexpr (K == 4) return max3f(v[0], v[1], fmaxf(v[2], v[3]));
+    if constexpr (K == 4) return max3f(v[0], v[1], fmaxf(v[2], v[3]));
     else if constexpr (K == 8) return max3f(max3f(v[0], v[1], v[2]), max3f(v[3], v[4], v[5]), fmaxf(v[6], v[7]));
     else
         return max3f(max3f(max3f(v[0], v[1], v[2]), max3f(v[3], v[4], v[5]), max3f(v[6], v[7], v[8])),
@@ -287,19 +287,13 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
                 {
                     const float *bx = stg + (o >> 5) * 1024;
                     const int w = o & 31;
-                    if constexpr (K >= 4) {
 #pragma unroll
-                        for (int q = 0; q < K / 4; ++q) {
-                            const float4 u = *reinterpret_cast<const float4 *>(bx + 4 * (((w >> 2) + q) ^ sw));
-                            x[4 * q] = u.x;
-                            x[4 * q + 1] = u.y;
-                            x[4 * q + 2] = u.z;
-                            x[4 * q + 3] = u.w;
-                        }
-                    } else {
-                        const float2 u = *reinterpret_cast<const float2 *>(bx + 4 * ((w >> 2) ^ sw) + (w & 3));
-                        x[0] = u.x;
-                        x[1] = u.y;
+                    for (int q = 0; q < K / 4; ++q) {
+                        const float4 u = *reinterpret_cast<const float4 *>(bx + 4 * (((w >> 2) + q) ^ sw));
+                        x[4 * q] = u.x;
+                        x[4 * q + 1] = u.y;
+                        x[4 * q + 2] = u.z;
+                        x[4 * q + 3] = u.w;
                     }
                 }
 
@@ -473,15 +467,132 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
             }
             return true;
         };
+        // One group of 32 rows step by step (short T_eff): Eqs 1-5 in double-single.  What a spike changes
+        // at the next step is known beforehand (T_eff >= 2: that step is refractory, its membrane 0), so a
+        // step t is computed as if t - 1 had none and corrected by it afterwards, and the serial chain
+        // through the decision, the adaptation and the threshold spans two steps instead of one.  State
+        // between steps: V(t-1) as computed, Sp = S[t-1], a(t-1), and rel, the steps from t on masked by
+        // spikes before t - 1.  Bound by instructions and that chain (1.7 warps per scheduler at 32768
+        // rows): 113 us with the chain through every step, 88 through two, 85 with the next quad's
+        // currents loaded ahead; V and a in packed arithmetic measured the same.
+        auto group_steps = [&]() -> bool {
+            const df beta{nr.beta_hi, nr.beta_lo}, p{nr.p_hi, nr.p_lo};
+            const float ch = nr.c_hi, cl = nr.c_lo, d = nr.d, th0 = nr.theta0;
+            const float dp = d * p.hi, tiny = 0x1p-19f * fabsf(th0);
+            const int T = (int)A.T, teff = nr.teff;
+            AlifState s0{0.0f, 0.0f, 0};
+            if (A.init && live) s0 = A.init[r];
+            int rel = s0.rem > 0 ? s0.rem : 0;
+            df V{rel > 0 ? 0.0f : s0.v, 0.0f}, a{s0.a, 0.0f};
+            bool Sp = false;
+            AlifState *ck = (A.ckpt && live) ? A.ckpt + r * A.nckpt : nullptr;
+            uint32_t *spw = A.spikes + (live ? r : 0) * A.nwords;
+            const int nw = (T + 31) >> 5;
+            auto entering = [&](int wd) {  // the state entering a word, as Eqs 1-5 have it
+                AlifState cs;
+                cs.v = Sp ? 0.0f : V.hi;
+                cs.a = (wd > 0 ? df_axpy(p, a, df{Sp ? 1.0f : 0.0f, 0.0f}) : a).hi;
+                cs.rem = Sp ? teff - 1 : max(rel, 0);
+                return cs;
+            };
+            const float *stg = nullptr;
+            for (int wd = 0; wd < nw; ++wd) {
+                if ((wd & (SPAN / 32 - 1)) == 0) {  // the word opens a stage
+                    if (wd > 0) {
+                        __syncwarp();
+                        fence_proxy_async_smem();
+                        ++consumed;
+                        issue();
+                    }
+                    const int st = consumed % NST;
+                    if (!mbar_wait_bounded(&bars[st], (consumed / NST) & 1u)) {
+                        report_timeout(A.status);
+                        return false;
+                    }
+                    stg = ring + st * (STAGE_BYTES / 4) + lane * 32;
+                }
+                if ((wd & 7) == 0 && ck) ck[wd / (ALIF_CKPT_STEPS / 32)] = entering(wd);
+                const float *bx = stg + (wd & (SPAN / 32 - 1)) * 1024;
+                const int nq = wd == nw - 1 ? (T - (wd << 5)) >> 2 : 8;  // T is a multiple of 4
+                uint32_t sword = 0;
+                float4 un = *reinterpret_cast<const float4 *>(bx + 4 * sw);
+#pragma unroll 1
+                for (int q = 0; q < nq; ++q) {
+                    const float4 u = un;
+                    un = *reinterpret_cast<const float4 *>(bx + 4 * (((q + 1) & 7) ^ sw));  // the next quad's
+                    const float x[4] = {u.x, u.y, u.z, u.w};
+                    const df Vq = V, aq = a;
+                    const bool Sq = Sp;
+                    const int relq = rel;
+                    unsigned sq = 0;
+                    bool near = wd + q == 0;  // the first steps have no step before them
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float xm = rel > 0 ? 0.0f : x[k];
+                        df I = two_prod(ch, xm);  // c I m (Eqs 2, 4)
+                        I.lo = __fmaf_rn(cl, xm, I.lo);
+                        const float ah = a.hi;
+                        const df Vt = df_axpy(beta, V, I);
+                        a = df_axpy(p, a, df{Sp ? 1.0f : 0.0f, 0.0f});
+                        // Eq 1 against theta = theta0 + d p a(t-1) (Eq 5 without a spike at t - 1).  The
+                        // FP32 difference is within 2^-21 (|theta| + theta0) of the double-single margin
+                        // (near theta, |V| is |theta|), so its sign is the margin's outside 2^-19 (...).
+                        const float thf = __fmaf_rn(dp, ah, th0), dz = Vt.hi - thf;
+                        const bool adm = rel <= 0 && !Sp;
+                        near = near || (adm && fabsf(dz) <= __fmaf_rn(0x1p-19f, fabsf(thf), tiny));
+                        rel = (Sp ? teff - 1 : rel) - 1;
+                        V = Sp ? df{0.0f, 0.0f} : Vt;
+                        Sp = adm && dz > 0.0f;
+                        if (Sp) sq |= 1u << k;
+                    }
+                    if (near) {  // the quad again, each margin in double-single
+                        Sp = Sq;
+                        sq = 0;
+                        V = Sp ? df{0.0f, 0.0f} : Vq;
+                        a = wd + q > 0 ? df_axpy(p, aq, df{Sp ? 1.0f : 0.0f, 0.0f}) : aq;
+                        rel = Sp ? teff - 1 : relq;
+#pragma unroll 1
+                        for (int k = 0; k < 4; ++k) {
+                            if (k > 0) {
+                                if (Sp) V = df{0.0f, 0.0f};
+                                a = df_axpy(p, a, df{Sp ? 1.0f : 0.0f, 0.0f});
+                                if (Sp) rel = teff - 1;
+                            }
+                            const float xk = k == 0 ? u.x : k == 1 ? u.y : k == 2 ? u.z : u.w;
+                            df I = two_prod(ch, xk);
+                            I.lo = __fmaf_rn(cl, xk, I.lo);
+                            if (rel > 0) I = df{0.0f, 0.0f};
+                            V = df_axpy(beta, V, I);
+                            const df dm = df_add(V, df_neg(df_add(df{th0, 0.0f}, df_mul_f(a, d))));
+                            Sp = rel <= 0 && dm.hi > 0.0f;
+                            if (rel <= 0 && fabsf(dm.hi) <= __fmaf_rn(0x1p-19f, fabsf(V.hi), tiny)) {
+                                ++n_exact;
+                                n_exact_spk += Sp;
+                            }
+                            rel -= 1;
+                            if (Sp) sq |= 1u << k;
+                        }
+                    }
+                    sword |= sq << (4 * q);
+                }
+                if (live) spw[wd] = sword;
+            }
+            __syncwarp();
+            fence_proxy_async_smem();
+            ++consumed;
+            issue();
+            if (A.fin && live) A.fin[r] = entering(nw);
+            return true;
+        };
         bool ok;
         if (tmin >= 16)
             ok = group(std::integral_constant<int, 16>{});
         else if (tmin >= 8)
             ok = group(std::integral_constant<int, 8>{});
-        else if (tmin >= 4)
+        else if (tmin >= 4)  // 32768 rows of 1000 steps: 82 us, by steps 88
             ok = group(std::integral_constant<int, 4>{});
-        else
-            ok = group(std::integral_constant<int, 2>{});
+        else  // 85 us, by Blocks of two steps 113 to 117 (and 103 without a spike)
+            ok = group_steps();
         dead = !ok;
         if (live) ++n_rows;
     }

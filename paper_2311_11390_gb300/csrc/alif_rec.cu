@@ -106,20 +106,6 @@ __device__ __forceinline__ void cp_async_wait() {
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// b v + x for double-single b, v, x: the product of the high parts split exactly (FMA), the
-// low-order terms added once (relative error about 2^-46); a shorter dependent chain than a
-// double-single product followed by a double-single sum
-__device__ __forceinline__ df df_axpy(df b, df v, df x) {
-    const float p = b.hi * v.hi;
-    const float e = fmaf(b.hi, v.hi, -p);
-    const df s = two_sum(p, x.hi);
-    float lo = e + s.lo;
-    lo = fmaf(b.hi, v.lo, lo);
-    lo = fmaf(b.lo, v.hi, lo);
-    lo += x.lo;
-    return quick_two_sum(s.hi, lo);
-}
-
 // MAXT: the CTA size the register budget is sized for (256: up to 255 registers a thread, for
 // clusters of at most 256 neurons per CTA; 1024 otherwise).  VW: floats per unit of the currents.
 template <int MAXT, int VW>

@@ -71,6 +71,20 @@ __device__ __forceinline__ df df_mul_f(df a, float b) {
     return quick_two_sum(p.hi, p.lo);
 }
 
+// b v + x for double-single b, v, x: the product of the high parts split exactly (FMA), the
+// low-order terms added once (relative error about 2^-46); a shorter dependent chain than a
+// double-single product followed by a double-single sum
+__device__ __forceinline__ df df_axpy(df b, df v, df x) {
+    const float p = b.hi * v.hi;
+    const float e = fmaf(b.hi, v.hi, -p);
+    const df s = two_sum(p, x.hi);
+    float lo = e + s.lo;
+    lo = fmaf(b.hi, v.lo, lo);
+    lo = fmaf(b.lo, v.hi, lo);
+    lo += x.lo;
+    return quick_two_sum(s.hi, lo);
+}
+
 // b^n by binary exponentiation (n >= 0).
 __device__ __forceinline__ df df_pow(df b, long long n) {
     df r = df{1.0f, 0.0f};
