@@ -145,8 +145,8 @@ int64_t alif_ckpt_count(int64_t T);
  *   ckpt     [B,N,alif_ckpt_count(T)] AlifState: state entering step 256k, or NULL
  *            (alif_backward needs it)
  *   final_state [B,N] AlifState state entering step T, or NULL
- * With B*N >= 32 x the SM count (and no traces), a lane takes a row and walks
- * it through Blocks of K <= T_eff steps (K = 16, 8, 4 or 2): the Block's
+ * With B*N >= 80 x the SM count (and no traces), a lane takes a row and walks
+ * it through Blocks of K <= T_eff steps (K = 16, 8 or 4; below, step by step): the Block's
  * no-reset membrane (Prop 1) from an input-only chain, its first crossing
  * (Prop 2, Eq 9), and the state carried to the next Block (Props 3-5).  With
  * fewer rows, or with traces, a warp takes a row: inside each 256- or 512-step
@@ -158,8 +158,8 @@ int64_t alif_ckpt_count(int64_t T);
  * FP32 margin lies within an error bound counted from the kernel's own
  * roundings are re-decided in double-single arithmetic from an exact anchor,
  * so the spikes equal the FP64 standard model's except at ties far below FP32
- * resolution.  I must be 4-byte aligned; 16-byte alignment with T % 4 == 0
- * enables the bulk-copy path (and is required for the lane layout). */
+ * resolution.  I must be 4-byte aligned; 16-byte alignment is required for the
+ * lane layout, and with T % 4 == 0 enables the bulk-copy path. */
 int alif_forward(int64_t B, int64_t N, int64_t T, const float *I,
                  const AlifNeuron *neurons, const AlifState *init,
                  uint32_t *spikes, float *v_trace, float *a_trace,
@@ -203,7 +203,7 @@ int alif_forward_window(int steps);
 
 /* Layout of alif_forward (host; a performance choice: the spikes are the same,
  * checkpoints and final states agree within FP32 rounding).  0, the default: a
- * lane per row when B * N >= 32 x the SM count, a warp per row otherwise.
+ * lane per row when B * N >= 80 x the SM count, a warp per row otherwise.
  * 1: a warp per row (the windows above).  2: a lane per row: each lane walks its
  * row through Blocks of K <= T_R steps (K = 8, 4 or 2 by the smallest T_eff of
  * the warp's 32 rows), at most one spike per Block (Section 3.1), with the

@@ -913,9 +913,12 @@ int launch_alif_forward(long long B, long long N, long long T, const float *I,
         cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
         if (g_sm_count <= 0) g_sm_count = 1;
     }
-    // a lane per row when the rows alone fill every SM's warp slots several times over (traces
-    // are written by the warp-per-row kernel); it declines calls it cannot stage with TMA
-    const bool lanes = g_fwd_layout == 2 || (g_fwd_layout == 0 && A.rows >= 32LL * g_sm_count);
+    // a lane per row when the rows alone fill the chip (traces are written by the warp-per-row kernel);
+    // it declines calls it cannot stage with TMA.  Its time hardly depends on the rows up to 32768, the
+    // warp-per-row kernel's is proportional to them; 2000 steps, us, lanes / warps at 8192, 12288 and
+    // 16384 rows: T_eff = 20 66 / 49, 69 / 66, 68 / 80; 10 76 / 50, 78 / 64, 78 / 81; 4 146 / 102,
+    // 146 / 146, 148 / 175; 2 109 / 103, 109 / 149, 109 / 175
+    const bool lanes = g_fwd_layout == 2 || (g_fwd_layout == 0 && A.rows >= 80LL * g_sm_count);
     if (lanes && !vtr && !atr) {
         bool declined = false;
         const int rc =

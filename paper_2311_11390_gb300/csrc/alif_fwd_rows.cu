@@ -22,6 +22,12 @@
 // Input: stages of [32 rows x 64 steps] (two 2-D TMA boxes of 32 x 32 floats, 128-byte swizzle)
 // in a three-deep ring per warp; a lane reads its own row's K steps with 16-byte loads, which
 // the swizzle spreads over distinct bank groups.
+// Where T is not a multiple of 4 (RAG) rows start at any 4-byte boundary, but four rows together are
+// a multiple of 16 bytes: the tensor is viewed as [rows / 4][4 T], a stage is four boxes of 8 such
+// super rows x 68 steps, one for each row of a super row from the boundary at or before its step, and
+// a lane shifts what it reads by its row's offset in registers.  The up to three rows past the last
+// super row are copied by their lanes, a stage ahead.  (The warp-per-row kernel took these calls: 32768 rows of
+// 1001 steps at T_eff = 2 187 -> 89 us, of 4001 steps at T_eff = 20 264 -> 150 us.)
 //
 // Exactness of the spike decisions, as in the warp-per-row kernel: the FP32 margin comes with an
 // error bound G, and a margin within G is re-decided in double-single arithmetic from the lane's
@@ -69,7 +75,14 @@ static_assert(SPAN % 32 == 0 && NBOX >= 1, "stages of whole boxes");
 constexpr int KMAX = 16;                       // longest Block
 // the ring, its barriers, the lanes' p^k tables (float2 [KMAX][32]) and beta^-r tables (float
 // [KMAX][32]), alignment of the swizzled ring
-constexpr int SMEM_BYTES = NST * STAGE_BYTES + NST * 8 + KMAX * 32 * 12 + 1024;
+// RAG: floats of a super row's box row (64 steps and up to 3 before them), bytes of a box and of a
+// stage; two stages keep as many warps on an SM
+constexpr int RPITCH = SPAN + 4, RBOX_BYTES = 8 * RPITCH * 4, RSTAGE_BYTES = 4 * RBOX_BYTES, RNST = 2;
+static_assert(RBOX_BYTES % 128 == 0 && RPITCH % 4 == 0, "boxes 128-byte aligned, rows 16-byte aligned");
+constexpr int TAIL_BYTES = 2 * 3 * RPITCH * 4;  // two stages of the rows past the last super row
+constexpr int smem_bytes(bool rag) {
+    return (rag ? RNST * (RSTAGE_BYTES + 8) + TAIL_BYTES : NST * (STAGE_BYTES + 8)) + KMAX * 32 * 12 + 1024;
+}
 
 struct Args {
     long long rows, N, T, nwords, nckpt, ngroups;
@@ -136,7 +149,19 @@ __device__ __forceinline__ df df_add_sloppy(df a, df b) {
     return quick_two_sum(s.hi, s.lo);
 }
 
+// K floats from y[sh], sh = 0..3 (K + 4 floats at y).
+template <int K>
+__device__ __forceinline__ void shifted(const float (&y)[K + 4], int sh, float (&x)[K]) {
+    float u[K + 2];
+#pragma unroll
+    for (int k = 0; k < K + 2; ++k) u[k] = (sh & 1) ? y[k + 1] : y[k];
+#pragma unroll
+    for (int k = 0; k < K; ++k) x[k] = (sh & 2) ? u[k + 2] : u[k];
+}
+
+template <bool RAG>
 __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CUtensorMap tm, const Args A) {
+    constexpr int NST = RAG ? RNST : fwdr::NST, STAGE_BYTES = RAG ? RSTAGE_BYTES : fwdr::STAGE_BYTES;
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     unsigned char *sm = smem_raw + (((raw + 1023u) & ~1023u) - raw);  // 128-byte swizzle: 1024-aligned boxes
@@ -146,6 +171,8 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
     float2 *ptab = reinterpret_cast<float2 *>(sm + NST * STAGE_BYTES + NST * 8);
     // beta^-r, 0 < r < K, of each lane's row at [r][lane]
     float *btab = reinterpret_cast<float *>(ptab + KMAX * 32);
+    // rows past the last super row, [2 stages][3 rows][RPITCH] (RAG)
+    float *tails = btab + KMAX * 32;
     const int lane = threadIdx.x;
     const long long ng = gridDim.x;
     if ((long long)blockIdx.x >= A.ngroups) return;
@@ -167,11 +194,17 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
                 const int st = issued % NST;
                 const uint32_t dst = smem_u32(ring) + st * STAGE_BYTES, bar = smem_u32(&bars[st]);
                 const int x = p_s * SPAN, y = (int)(p_g * 32);
-                // boxes holding steps < T only (no box lies wholly outside the tensor)
-                const long long left = A.T - x;
-                const int nbx = left >= SPAN ? NBOX : (int)((left + 31) / 32);
-                mbar_arrive_expect_tx(&bars[st], nbx * BOX_BYTES);
-                for (int b = 0; b < nbx; ++b) tma_load_2d_u(dst + b * BOX_BYTES, &tm, x + 32 * b, y, bar);
+                if (RAG) {
+                    mbar_arrive_expect_tx(&bars[st], STAGE_BYTES);
+                    for (int j = 0; j < 4; ++j)
+                        tma_load_2d_u(dst + j * RBOX_BYTES, &tm, (int)((j * A.T) & ~3LL) + x, y / 4, bar);
+                } else {
+                    // boxes holding steps < T only (no box lies wholly outside the tensor)
+                    const long long left = A.T - x;
+                    const int nbx = left >= SPAN ? NBOX : (int)((left + 31) / 32);
+                    mbar_arrive_expect_tx(&bars[st], nbx * BOX_BYTES);
+                    for (int b = 0; b < nbx; ++b) tma_load_2d_u(dst + b * BOX_BYTES, &tm, x + 32 * b, y, bar);
+                }
             }
             ++issued;
             if (++p_s == nstg) {
@@ -183,14 +216,48 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
     issue();
 
     const int sw = lane & 7;  // this lane's row in the swizzle pattern
+    // lane -> row of the group; RAG: 8 lanes take one row each of 8 super rows, whose 16-byte reads fall in
+    // distinct bank groups
+    auto row_of = [&](int l) { return RAG ? 4 * (l & 7) + (l >> 3) : l; };
+    // this lane's row in a stage (floats), and its offset there
+    const int srow = RAG ? (lane >> 3) * (RBOX_BYTES / 4) + (lane & 7) * RPITCH : lane * 32;
+    const int sh = RAG ? (int)(((lane >> 3) * A.T) & 3) : 0;
     unsigned n_exact = 0, n_exact_spk = 0, n_rows = 0;
     bool dead = false;
     for (long long g = blockIdx.x; g < A.ngroups && !dead; g += ng) {
-        const long long r = g * 32 + lane;
+        const long long r = g * 32 + row_of(lane);
         const bool live = r < A.rows;
         const AlifNeuron nr = A.nrn[(live ? r : g * 32) % A.N];
         const int tmin = (int)__reduce_min_sync(FULL, live ? (unsigned)nr.teff : 0x7fffffffu);
 
+        // RAG: the rows past the last super row have no box; their lanes copy them a stage ahead
+        const bool tail = RAG && live && r >= (A.rows & ~3LL);
+        float *trow = tails + (tail ? (int)(r & 3) : 0) * RPITCH;  // two stages, 3 RPITCH floats apart
+        int f_t = 0;  // first step of the next stage to be waited for
+        auto copy_tail = [&]() {
+            float *dst = trow + ((f_t / SPAN) & 1) * 3 * RPITCH + sh;
+            const float *src = A.I + r * A.T + f_t;
+            const int n = A.T - f_t < SPAN ? (int)(A.T - f_t) : SPAN;
+            for (int k = 0; k < n; ++k)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst + k)), "l"(src + k) : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        if (tail) copy_tail();
+        auto wait_stage = [&](const float *&stg) -> bool {
+            const int st = consumed % NST;
+            if (!mbar_wait_bounded(&bars[st], (consumed / NST) & 1u)) {
+                report_timeout(A.status);
+                return false;
+            }
+            stg = ring + st * (STAGE_BYTES / 4) + srow;
+            f_t += SPAN;
+            if (tail) {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+                stg = trow + ((f_t / SPAN - 1) & 1) * 3 * RPITCH;
+                if (f_t < A.T) copy_tail();
+            }
+            return true;
+        };
         // One group of 32 rows with K-step Blocks; false if a stage never arrived.
         auto group = [&](auto ktag) -> bool {
             constexpr int K = decltype(ktag)::value;
@@ -253,15 +320,6 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
 
             // ---- staging: the stage holding the current word; a lane's K inputs of a Block
             const float *stg = nullptr;  // this lane's box row in that stage
-            auto wait_stage = [&]() -> bool {
-                const int st = consumed % NST;
-                if (!mbar_wait_bounded(&bars[st], (consumed / NST) & 1u)) {
-                    report_timeout(A.status);
-                    return false;
-                }
-                stg = ring + st * (STAGE_BYTES / 4) + lane * 32;
-                return true;
-            };
             auto release_stage = [&]() {  // the stage's inputs are all in registers
                 __syncwarp();
                 fence_proxy_async_smem();
@@ -284,7 +342,22 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
                 constexpr bool FULLB = decltype(fulltag)::value;
                 const int cnt = FULLB ? K : cnt_in;
                 float x[K];
-                {
+                if constexpr (RAG) {
+                    float y[K + 4];
+#pragma unroll
+                    for (int q = 0; q < K / 4 + 1; ++q) {
+                        const float4 u = *reinterpret_cast<const float4 *>(stg + o + 4 * q);
+                        y[4 * q] = u.x;
+                        y[4 * q + 1] = u.y;
+                        y[4 * q + 2] = u.z;
+                        y[4 * q + 3] = u.w;
+                    }
+                    shifted<K>(y, sh, x);
+                    if (!FULLB) {  // the next row's steps follow
+#pragma unroll
+                        for (int k = 0; k < K; ++k) x[k] = k < cnt ? x[k] : 0.0f;
+                    }
+                } else {
                     const float *bx = stg + (o >> 5) * 1024;
                     const int w = o & 31;
 #pragma unroll
@@ -389,7 +462,7 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
                             thx.hi = __shfl_sync(FULL, thx.hi, Lx);
                             thx.lo = __shfl_sync(FULL, thx.lo, Lx);
                             const int tg = tb + kx;
-                            const df Vx = exact_membrane<false>(A.I + (g * 32 + Lx) * A.T, at, avh, avl, tg, bh, bl,
+                            const df Vx = exact_membrane<false>(A.I + (g * 32 + row_of(Lx)) * A.T, at, avh, avl, tg, bh, bl,
                                                                 ch, cl, lane);
                             if (lane == Lx) {
                                 ++n_exact;
@@ -426,11 +499,11 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
             constexpr int WPS = SPAN / 32;  // words per stage
             constexpr int BPW = 32 / K;     // Blocks per word
             const int nfw = T >> 5;
-            if (!wait_stage()) return false;
+            if (!wait_stage(stg)) return false;
             for (int wd = 0; wd < nfw; ++wd) {
                 if (wd > 0 && (wd & (WPS - 1)) == 0) {  // the word opens the next stage
                     release_stage();
-                    if (!wait_stage()) return false;
+                    if (!wait_stage(stg)) return false;
                 }
                 if ((wd & 7) == 0) checkpoint(wd << 5);
                 const int ow = (wd & (WPS - 1)) << 5;  // the word's first step within the stage
@@ -448,7 +521,7 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
             if (tt < T) {
                 if (nfw > 0 && (nfw & (WPS - 1)) == 0) {
                     release_stage();
-                    if (!wait_stage()) return false;
+                    if (!wait_stage(stg)) return false;
                 }
                 if ((nfw & 7) == 0) checkpoint(tt);
                 const int ow = (nfw & (WPS - 1)) << 5;
@@ -504,28 +577,31 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
                         ++consumed;
                         issue();
                     }
-                    const int st = consumed % NST;
-                    if (!mbar_wait_bounded(&bars[st], (consumed / NST) & 1u)) {
-                        report_timeout(A.status);
-                        return false;
-                    }
-                    stg = ring + st * (STAGE_BYTES / 4) + lane * 32;
+                    if (!wait_stage(stg)) return false;
                 }
                 if ((wd & 7) == 0 && ck) ck[wd / (ALIF_CKPT_STEPS / 32)] = entering(wd);
-                const float *bx = stg + (wd & (SPAN / 32 - 1)) * 1024;
-                const int nq = wd == nw - 1 ? (T - (wd << 5)) >> 2 : 8;  // T is a multiple of 4
+                const float *bx = stg + (wd & (SPAN / 32 - 1)) * (RAG ? 32 : 1024);
+                auto quad = [&](int q) { return *reinterpret_cast<const float4 *>(bx + 4 * (RAG ? q : (q & 7) ^ sw)); };
+                const int nst = wd == nw - 1 ? T - (wd << 5) : 32;  // steps of the word
                 uint32_t sword = 0;
-                float4 un = *reinterpret_cast<const float4 *>(bx + 4 * sw);
+                float4 un = quad(0);
 #pragma unroll 1
-                for (int q = 0; q < nq; ++q) {
-                    const float4 u = un;
-                    un = *reinterpret_cast<const float4 *>(bx + 4 * (((q + 1) & 7) ^ sw));  // the next quad's
+                for (int q = 0; 4 * q < nst; ++q) {
+                    float4 u = un;
+                    un = quad(q + 1);  // the next quad's
+                    if constexpr (RAG) {
+                        const float y[8] = {u.x, u.y, u.z, u.w, un.x, un.y, un.z, un.w};
+                        float v[4];
+                        shifted<4>(y, sh, v);
+                        u = make_float4(v[0], v[1], v[2], v[3]);
+                    }
                     const float x[4] = {u.x, u.y, u.z, u.w};
                     const df Vq = V, aq = a;
                     const bool Sq = Sp;
                     const int relq = rel;
                     unsigned sq = 0;
-                    bool near = wd + q == 0;  // the first steps have no step before them
+                    const int kn = RAG ? min(nst - 4 * q, 4) : 4;  // the row's last quad may be partial
+                    bool near = wd + q == 0 || kn < 4;             // the first steps have no step before them
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const float xm = rel > 0 ? 0.0f : x[k];
@@ -552,7 +628,7 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
                         a = wd + q > 0 ? df_axpy(p, aq, df{Sp ? 1.0f : 0.0f, 0.0f}) : aq;
                         rel = Sp ? teff - 1 : relq;
 #pragma unroll 1
-                        for (int k = 0; k < 4; ++k) {
+                        for (int k = 0; k < kn; ++k) {
                             if (k > 0) {
                                 if (Sp) V = df{0.0f, 0.0f};
                                 a = df_axpy(p, a, df{Sp ? 1.0f : 0.0f, 0.0f});
@@ -620,7 +696,8 @@ __global__ void __launch_bounds__(32) fwd_rows_kernel(const __grid_constant__ CU
 static int g_sm_count_rows = 0;
 
 // Row-per-lane forward: the launch's status.  *declined is set (nothing launched) when the input
-// cannot be staged with TMA (T % 4 != 0, I not 16-byte aligned, or the tensor map is rejected);
+// cannot be staged with TMA (I not 16-byte aligned, T % 4 != 0 with very few steps, or the tensor map
+// is rejected);
 // the caller then uses the warp-per-row kernel.
 int launch_alif_forward_rows(long long rows, long long N, long long T, const float *I, const AlifNeuron *nrn,
                              const AlifState *init, uint32_t *spikes, AlifState *ckpt, AlifState *fin,
@@ -628,10 +705,12 @@ int launch_alif_forward_rows(long long rows, long long N, long long T, const flo
     using namespace fwdr;
     *declined = true;
     // step indices (plus a refractory span of at most 1e6 steps) stay within int32
-    if (T % 4 != 0 || ((uintptr_t)I & 15u) != 0 || T >= (1LL << 30) || rows >= (1LL << 31)) return 0;
+    if (((uintptr_t)I & 15u) != 0 || T >= (1LL << 30) || rows >= (1LL << 31)) return 0;
+    const bool rag = T % 4 != 0;
+    if (rag && (T < SPAN || T >= (1LL << 28) || rows < 4)) return 0;  // box coordinates up to 4 T
     CUtensorMap tm;
     memset(&tm, 0, sizeof tm);
-    if (make_rowmajor_map(&tm, I, rows, T) != 0) return 0;
+    if ((rag ? make_super_rows_map(&tm, I, rows / 4, T, RPITCH) : make_rowmajor_map(&tm, I, rows, T)) != 0) return 0;
     *declined = false;
     Args A;
     memset(&A, 0, sizeof A);
@@ -655,19 +734,20 @@ int launch_alif_forward_rows(long long rows, long long N, long long T, const flo
         cudaDeviceGetAttribute(&g_sm_count_rows, cudaDevAttrMultiProcessorCount, dev);
         if (g_sm_count_rows <= 0) g_sm_count_rows = 1;
     }
-    static int occ = 0;
-    const void *fn = (const void *)fwd_rows_kernel;
+    static int occs[2] = {0, 0};
+    const void *fn = rag ? (const void *)fwd_rows_kernel<true> : (const void *)fwd_rows_kernel<false>;
+    int &occ = occs[rag];
     if (occ == 0) {
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(rag));
         int n = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, 32, SMEM_BYTES);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, 32, smem_bytes(rag));
         occ = n > 0 ? n : 1;
     }
     const long long cap = (long long)g_sm_count_rows * occ;
     const int grid = (int)(A.ngroups < cap ? A.ngroups : cap);
     if (grid <= 0) return 0;
     void *args[] = {&tm, &A};
-    return (int)cudaLaunchKernel(fn, dim3(grid), dim3(32), args, SMEM_BYTES, stream);
+    return (int)cudaLaunchKernel(fn, dim3(grid), dim3(32), args, smem_bytes(rag), stream);
 }
 
 }  // namespace alif

@@ -61,6 +61,22 @@ inline int make_rowmajor_map(CUtensorMap *map, const float *I, long long rows, l
     return r == CUDA_SUCCESS ? 0 : -2;
 }
 
+// FP32 currents [4 n4, T] with rows of any length, viewed as n4 super rows of four rows (4 T floats, a
+// multiple of 16 bytes); one box is 8 super rows x `width` floats, unswizzled.  Returns 0, -1 (no
+// encoder) or -2 (rejected: I must be 16-byte aligned).
+inline int make_super_rows_map(CUtensorMap *map, const float *I, long long n4, long long T, unsigned width) {
+    auto enc = tensor_map_encoder();
+    if (!enc) return -1;
+    const cuuint64_t dims[2] = {(cuuint64_t)T * 4, (cuuint64_t)n4};
+    const cuuint64_t strides[1] = {(cuuint64_t)T * 16};
+    const cuuint32_t box[2] = {width, 8};
+    const cuuint32_t estr[2] = {1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(I), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? 0 : -2;
+}
+
 // FP32 currents as [B, N, T]; one box is 32 rows x 16 steps of one batch element (64-byte
 // swizzle), clipped at N and T.  Returns 0, -1 (no encoder) or -2 (rejected: I must be 16-byte
 // aligned and T a multiple of 4).
