@@ -27,7 +27,7 @@ __device__ __forceinline__ float warp_sum(float x) {
 // n[b,k] = sum_t w[t] S[b,k,t] and o[b,c] = sum_k W[c,k] n[b,k] + bias_c w_sum: one block per batch
 // element, a warp per row, lanes over its words, then a warp per output, lanes over the inputs.  Bound by
 // latency: with a kernel for each sum and a thread per output 27 us at B = 128, K = 256, C = 20, T = 1000,
-// now @F.
+// now 13.
 __global__ void forward_kernel(long long K, long long C, long long T, long long nwords, const uint32_t *__restrict__ S,
                                const float *__restrict__ w, const float *__restrict__ W,
                                const float *__restrict__ bias, float w_sum, float *n, float *o) {
@@ -99,7 +99,7 @@ __device__ __forceinline__ void grad_w(long long e, long long B, long long K, lo
 
 // Both gradients in one launch: the first nw blocks take grad_w's elements (a serial sum over the batch,
 // hidden behind the writes of the others), the rest grad_spikes' rows.  As two kernels 27 + 30 us at
-// B = 128, K = 256, C = 20, T = 1000, now @B (the 131 MB written take 19).
+// B = 128, K = 256, C = 20, T = 1000, now 37 (the 131 MB written take 19).
 __global__ void __launch_bounds__(256, 8) backward_kernel(unsigned nw, long long B, long long K, long long C, long long T,
                                 const float *__restrict__ W, const float *__restrict__ g_o,
                                 const float *__restrict__ w, const float *__restrict__ n, float w_sum, float *gS,
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256, 8) backward_kernel(unsigned nw, long long
 }
 
 // Mean softmax cross-entropy: one block, a warp per row (a thread per row took 14 us at B = 128, C = 20,
-// now @C); the losses are summed in double, lanes over the rows, then a fixed tree.
+// now 10.5); the losses are summed in double, lanes over the rows, then a fixed tree.
 __global__ void ce_kernel(long long B, long long C, const float *__restrict__ o, const int32_t *__restrict__ y,
                           float *loss, float *g_o, float *row_loss) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
