@@ -676,15 +676,21 @@ def run_ours(args, rank, world, local_rank):
     steps_per_rank = B * N * T
     value = steps_per_rank * world / (ms_step / 1e3)
     kern_ms = {n: statistics.mean(a.elapsed_time(b) for a, b in ev[n]) for n in names if ev[n]}
-    launches_per_step = (1 if has_proj else 0) + 1 + 2  # projection, forward, backward + batch reduction
+    # projection (density sample, event lists, sums and the tensor-core kernel, which leaves the sparse tiles
+    # alone; that kernel only for small products), forward, backward (its fast-membrane follow-up at T % 16 == 0)
+    # and batch reduction
+    sparse = has_proj and alif.lib().syn_project_workspace_size(B, Nin, N, T) > 0
+    launches_per_step = (4 if sparse else int(has_proj)) + 1 + (3 if T % 16 == 0 else 2)
 
     # ---- roofline of the dominant kernel (algorithmic bytes or flops per launch)
     pk, pk_kind = peaks()
     alg = {
         "alif_forward": ("hbm", steps_per_rank * (4 + 1 / 8 + 12 / 256)),
         "alif_backward": ("hbm", steps_per_rank * (4 + 4 + 4 + 1 / 8 + 12 / 256)),
-        # dense split-BF16 contraction: 2 flops x 2 terms per weight and (b, t)
-        "syn_project": ("tensor", 4.0 * N * Nin * T * B),
+        # sums over the active inputs write I and read the raster and the weights; the dense split-BF16
+        # contraction takes 2 flops x 2 terms per weight and (b, t)
+        "syn_project": ("hbm", steps_per_rank * 4 + B * Nin * ((T + 31) // 32) * 4 + N * Nin * 4) if sparse
+        else ("tensor", 4.0 * N * Nin * T * B),
     }
     dom = max(kern_ms, key=kern_ms.get)
     bound, work = alg[dom]
@@ -706,8 +712,8 @@ def run_ours(args, rank, world, local_rank):
     roof["hbm_frac_per_block_state"] = {k: (alg_s[k] / (kern_ms[k] / 1e3) / 1e9) / pk["hbm_gbs"] for k in kern_ms
                                      if k in alg_s}
 
-    # ---- the event-driven projection on the same step (a separate line; the step above
-    # keeps the tensor-core projection)
+    # ---- the exact-weight event projection on the same step (a separate line; the step above
+    # keeps syn_project)
     extra = {}
     if has_proj and getattr(L, "syn_project_events", None) is not None:
         Wt_dev = alif.transpose_weights(W_dev)
@@ -724,11 +730,11 @@ def run_ours(args, rank, world, local_rank):
         ev_ms = max_over_ranks(e0.elapsed_time(e1) / reps, world, dev)
         step_ev = ev_ms + kern_ms["alif_forward"] + kern_ms["alif_backward"]
         extra["event_projection"] = {
-            "kernel_ms": ev_ms, "tensor_core_kernel_ms": kern_ms["syn_project"],
+            "kernel_ms": ev_ms, "projection_kernel_ms": kern_ms["syn_project"],
             "hbm_frac_of_output_write": (steps_per_rank * 4 / (ev_ms / 1e3) / 1e9) / pk["hbm_gbs"],
             "step_ms": step_ev, "value": steps_per_rank * world / (step_ev / 1e3),
-            "kernel": "event-driven: bias + sum of the active inputs' FP32 weights, per (batch, 32-step chunk) "
-                      "event lists in shared memory, deterministic order"}
+            "kernel": "event-driven: bias + sum of the active inputs' FP32 weights, event lists built once per "
+                      "call, deterministic order"}
         del I_ev, Wt_dev
 
     # ---- the projection fused into the block forward (currents summed inside the forward from the
@@ -778,10 +784,9 @@ def run_ours(args, rank, world, local_rank):
             "achieved_gbs": pb_bytes / (pb_ms / 1e3) / 1e9,
             "hbm_frac": pb_bytes / (pb_ms / 1e3) / 1e9 / pk["hbm_gbs"],
             "input_spikes": int(w.S_in.sum()),
-            "kernel": "dL/dW = sum_b,t dL/dI S^T and dL/dbias, event-driven (per batch element and 16-row "
-                      "tile, dL/dI staged step-major in 512-step chunks, one thread per input walking its "
-                      "spikes and adding the staged columns in registers), partials summed over the batch "
-                      "in a fixed order"}
+            "kernel": "dL/dW = sum_b,t dL/dI S^T and dL/dbias, event-driven (event lists of the raster built once "
+                      "per call, each neuron tile adding its staged columns of dL/dI), partials joined in a "
+                      "fixed order"}
 
     # ---- the same workload as a recurrent layer (W_rec, latency D = T_R): a separate line
     if has_proj and not args.no_rec and getattr(L, "alif_forward_recurrent", None) is not None:
@@ -942,7 +947,8 @@ def run_ours(args, rank, world, local_rank):
                                    "T=%d, DT=0.1 ms, ARP=%g ms (T_R=%d)" % (B, T, args.arp, alif.tr(0.1, args.arp)),
                        "global_batch": B * world, "seq_len": T, "parallelism": f"dp{world} (independent rows)",
                        "l2": "inputs larger than L2 (I, dL/dS: %.1f GB each)" % (steps_per_rank * 4 / 1e9),
-                       "projection": "tcgen05 split-BF16" if has_proj else "not in the loaded library (currents precomputed)"},
+                       "projection": ("split-BF16 weights, sums over the active inputs (tcgen05 for dense tiles)"
+                                      if sparse else "tcgen05 split-BF16") if has_proj else "not in the loaded library (currents precomputed)"},
             "roofline": roof, "cpu_baseline": cpu, "e2e": e2e, "e2e_spikes_only": e2e_spikes, "gpu_launches": launches_per_step * args.steps,
             "clocks": clk.summary(), **extra}
     line["targets"] = targets_summary(line)  # last, so the end of the printed line carries it
