@@ -87,14 +87,15 @@ __device__ __forceinline__ void mma_bf16(uint32_t d, uint64_t a, uint64_t b, uin
 __device__ __forceinline__ void tc_fence_before() { umma::fence_before(); }
 __device__ __forceinline__ void tc_fence_after() { umma::fence_after(); }
 
-template <bool WORDS_TMA>
+// LIST: only the tiles listed at A.dense (a run-time test in every tile's walk cost calls without a list 1 %)
+template <bool WORDS_TMA, bool LIST>
 __global__ void __launch_bounds__(THREADS, 1)
     proj_kernel(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
                 const __grid_constant__ CUtensorMap tm_s, const Args A) {
     extern __shared__ unsigned char smem_raw[];
-    const uint32_t *dense = A.dense && !__ldg(A.dense + 1) ? A.dense + 64 : nullptr;
-    const long long tiles = dense ? (long long)__ldg(A.dense) * A.tiles_m : A.tiles;
-    if (blockIdx.x >= tiles) return;
+    const uint32_t *dense = LIST && !__ldg(A.dense + 1) ? A.dense + 64 : nullptr;
+    const long long tiles = LIST && dense ? (long long)__ldg(A.dense) * A.tiles_m : A.tiles;
+    if (LIST && blockIdx.x >= tiles) return;
     // 1024-byte aligned base for the swizzled tiles
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     const int nk = A.nk;
     auto tile_coords = [&](long long tile, int &m0, long long &t0, long long &b) {
         const int mt = (int)(tile % A.tiles_m);
-        const long long at = tile / A.tiles_m, rest = dense ? (long long)__ldg(dense + at) : at;
+        const long long at = tile / A.tiles_m, rest = LIST && dense ? (long long)__ldg(dense + at) : at;
         m0 = mt * BM;
         t0 = (rest % A.tiles_t) * BN;
         b = rest / A.tiles_t;
@@ -475,19 +476,17 @@ int launch_syn_project(long long B, long long Nin, long long N, long long T, con
     const bool words_tma = (A.nwin % 4 == 0) && ((reinterpret_cast<uintptr_t>(S) & 15u) == 0) &&
                            make_words_map(&ms, S, B * Nin, A.nwin) == 0;
     if (!words_tma) memset(&ms, 0, sizeof ms);
-    static bool attr[2] = {false, false};
-    if (!attr[words_tma]) {
-        if (words_tma)
-            cudaFuncSetAttribute(proj_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        else
-            cudaFuncSetAttribute(proj_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-        attr[words_tma] = true;
-    }
-    if (words_tma)
-        proj_kernel<true><<<grid, THREADS, SMEM_BYTES, stream>>>(mh, ml, ms, A);
-    else
-        proj_kernel<false><<<grid, THREADS, SMEM_BYTES, stream>>>(mh, ml, ms, A);
-    return (int)cudaGetLastError();
+    static bool attr[4] = {false, false, false, false};
+    auto go = [&](auto kernel, int slot) -> int {
+        if (!attr[slot]) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+            attr[slot] = true;
+        }
+        kernel<<<grid, THREADS, SMEM_BYTES, stream>>>(mh, ml, ms, A);
+        return (int)cudaGetLastError();
+    };
+    if (dense) return words_tma ? go(proj_kernel<true, true>, 3) : go(proj_kernel<false, true>, 2);
+    return words_tma ? go(proj_kernel<true, false>, 1) : go(proj_kernel<false, false>, 0);
 }
 
 }  // namespace alif

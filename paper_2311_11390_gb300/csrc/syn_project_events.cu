@@ -98,7 +98,8 @@ struct Args {
     const uint32_t *dense;  // NULL or dense[1]: every chunk; else those of dense[0] tiles, listed from dense[64]
 };
 
-template <int NPT>
+// LIST: only the chunks of the tiles listed at A.dense
+template <int NPT, bool LIST>
 __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args A) {
     using C = Cfg<NPT>;
     constexpr int THREADS = C::THREADS, WARPS = C::WARPS, WPT = C::WPT, ACC_STRIDE = C::ACC_STRIDE;
@@ -109,8 +110,8 @@ __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args
     int *off = pos + GROUPS * 32;                                                  // [33] first event of step t
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // units are chunks; with a list, a tile's eight in order (those past T are passed over)
-    const uint32_t *dense = A.dense && !__ldg(A.dense + 1) ? A.dense + 64 : nullptr;
-    const long long units = dense ? 8LL * __ldg(A.dense) : A.B * A.nwords;
+    const uint32_t *dense = LIST && !__ldg(A.dense + 1) ? A.dense + 64 : nullptr;
+    const long long units = LIST && dense ? 8LL * __ldg(A.dense) : A.B * A.nwords;
     const long long tiles_t = (A.nwords + 7) / 8;
     const int nblk = (int)((A.Nin + IN_BLOCK - 1) / IN_BLOCK);
     for (long long nb = 0; nb < A.N; nb += NB_BLOCK) {
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args
         const bool any_live = live[0];
         for (long long u = blockIdx.x; u < units; u += gridDim.x) {
             long long b = u / A.nwords, c = u % A.nwords;
-            if (dense) {
+            if (LIST && dense) {
                 const long long tile = __ldg(dense + (u >> 3));
                 b = tile / tiles_t;
                 c = (tile - b * tiles_t) * 8 + (u & 7);
@@ -301,7 +302,7 @@ int launch_syn_project_events(long long B, long long Nin, long long N, long long
     const long long units = B * A.nwords;
     if (units == 0 || N == 0) return 0;
     static int sms = 0;
-    static bool attr[3] = {false, false, false};
+    static bool attr[6] = {false, false, false, false, false, false};
     if (!sms) {
         int dev = 0;
         cudaGetDevice(&dev);
@@ -321,9 +322,14 @@ int launch_syn_project_events(long long B, long long Nin, long long N, long long
         kernel<<<grid, threads, smem, st>>>(A);
         return (int)cudaGetLastError();
     };
-    if (npt == 4) return go(events_kernel<4>, Cfg<4>::SMEM_BYTES, Cfg<4>::THREADS, 2);
-    if (npt == 2) return go(events_kernel<2>, Cfg<2>::SMEM_BYTES, Cfg<2>::THREADS, 1);
-    return go(events_kernel<1>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 0);
+    if (dense) {
+        if (npt == 4) return go(events_kernel<4, true>, Cfg<4>::SMEM_BYTES, Cfg<4>::THREADS, 5);
+        if (npt == 2) return go(events_kernel<2, true>, Cfg<2>::SMEM_BYTES, Cfg<2>::THREADS, 4);
+        return go(events_kernel<1, true>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 3);
+    }
+    if (npt == 4) return go(events_kernel<4, false>, Cfg<4>::SMEM_BYTES, Cfg<4>::THREADS, 2);
+    if (npt == 2) return go(events_kernel<2, false>, Cfg<2>::SMEM_BYTES, Cfg<2>::THREADS, 1);
+    return go(events_kernel<1, false>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 0);
 }
 
 }  // namespace alif
