@@ -1,3 +1,4 @@
+#include <cmath>
 // Weight and bias gradients of the synaptic projection over sparse rasters:
 //     g_W[i, j] = sum_{b,t} g_I[b, i, t] S[b, j, t],   g_bias[i] = sum_{b,t} g_I[b, i, t].
 // Every input spike adds one column of g_I to its input's row of g_W^T.
@@ -423,6 +424,9 @@ __global__ void __launch_bounds__(1024) gw_join_kernel(long long N, int Nin, int
     }
 }
 
+// Active inputs per step above which a raster is left to the other kernel (its events would not fit the records).
+inline float active_limit(int Nin) { return 7.0f * ((float)rows_of(Nin) - Nin / 4.0f) / CH; }
+
 inline int sm_count() {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
@@ -442,12 +446,22 @@ size_t syn_grad_weights_ws(long long B, long long Nin, long long N, long long T)
     // 41 us, at 128 x 256 -> 256 x 1000 (8e9) 77 to 113 against 142 to 285, at 1 x 512 -> 2000 x 16384 (2e10)
     // 103 against 129.  Many inputs at high rates do not fit the lists; there the other kernel's call
     // becomes 20 us longer, so it has to be a long one.
+    // The other kernel walks a batch element's 512-step chunks in series, a CTA for 16 neurons and 1024
+    // inputs, so its time goes with waves of CTAs x chunks (3 to 6 us each); from 12 of those the lists pay
+    // whatever the product (us, that / this): 22 x 113 -> 270 x 7500 (3 x 15) 144 / 91, 30 x 64 -> 600 x 4000
+    // (8 x 8) 232 / 99, 1 x 512 -> 200 x 16000 (1 x 32) 138 / 52, 17 x 700 -> 276 x 3900 at 21 active inputs a
+    // step (3 x 8) 310 / 142; not for 12 x 512 -> 289 x 2393 (2 x 5) 58 / 60 or 4 x 1000 -> 1024 x 1500
+    // (2 x 3) 66 / 79.  Where a raster of 3.5 % activity would not fit the lists, from 36.
+    const int sms = sm_count();
+    if (!sms) return 0;
+    const double ctas = (double)B * (double)((N + 15) / 16) * (double)((Nin + 1023) / 1024);
+    const double least = active_limit((int)Nin) >= 0.035f * (float)Nin ? 12.0 : 36.0;
+    const bool many = std::ceil(ctas / sms) * (double)((T + 511) / 512) >= least;
     const double wide = Nin > 350 ? Nin / 350.0 : 1.0;
-    if ((double)B * (double)Nin * (double)N * (double)T < 8e9 * wide) return 0;
+    if (!many && (double)B * (double)Nin * (double)N * (double)T < 8e9 * wide) return 0;
     const long long units = B * ((T + CH - 1) / CH), tiles = (N + NT - 1) / NT;
     if (units > (1LL << 24) || tiles > (1LL << 20)) return 0;
-    const int sms = sm_count();
-    return sms ? layout(units, tiles, ranges_for(tiles, units, sms), (int)Nin, nullptr, nullptr) : 0;
+    return layout(units, tiles, ranges_for(tiles, units, sms), (int)Nin, nullptr, nullptr);
 }
 
 // g_W and g_bias of a sparse raster; *flags (device): flags[1] set where it is too dense for the
@@ -462,7 +476,7 @@ int launch_syn_grad_weights(long long B, long long Nin, long long N, long long T
     A.ranges = ranges_for(A.tiles, A.units, sms);
     layout(A.units, A.tiles, A.ranges, (int)Nin, work, &A.ws);
     *flags = A.ws.flag;
-    int rc = launch_density_sample(S, B * Nin * nwin, Nin, 7.0f * ((float)rows_of((int)Nin) - Nin / 4.0f) / CH, A.ws.flag, st);
+    int rc = launch_density_sample(S, B * Nin * nwin, Nin, active_limit((int)Nin), A.ws.flag, st);
     if (rc) return rc;
     cudaError_t e = cudaFuncSetAttribute(gw_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (HEAD + 16 * MAX_ROWS));
     if (e != cudaSuccess) return (int)e;
