@@ -51,8 +51,9 @@ __host__ __device__ constexpr int rec_of(int Nin) { return HEAD + 16 * rows_of(N
 __host__ __device__ constexpr int smem_of(int Nin) { return GT_BYTES + sums_bytes(Nin) + 2 * rec_of(Nin) + 64; }
 static_assert(smem_of(MAX_NIN) <= SMEM && rows_of(MAX_NIN) >= 1000, "10 spikes a step fit at any Nin");
 
-// Workspace: [1] whether the raster is too dense for the lists; from byte 256 the units' sizes
-// (groups | rows << 16), their records, the ranges' sums [range][tile][input][32] and of g_I itself [range][tile][32].
+// Workspace: [1] whether a sample of the raster is too dense for the lists, [2] whether a unit's list
+// did not fit (two words: the lists kernel, whose blocks all decide by [1] whether to run, writes [2]);
+// from byte 256 the units' sizes (groups | rows << 16), their records, the ranges' sums [range][tile][input][32] and of g_I itself [range][tile][32].
 struct Work {
     uint32_t *flag, *count;
     unsigned char *rec;
@@ -82,6 +83,9 @@ inline int ranges_for(long long tiles, long long units, int sms) {
     }
     return best;
 }
+
+// Whether the other kernel has to run: after the lists kernel, when nobody writes the flags any more.
+__device__ __forceinline__ bool too_dense(const uint32_t *flag) { return __ldg(flag + 1) | __ldg(flag + 2); }
 
 // One CTA per 1024 steps (two units) of a batch element: a warp holds a 32nd of the rows, a lane the
 // word of 32 steps, so that the raster is read in whole lines.
@@ -205,7 +209,7 @@ __global__ void __launch_bounds__(1024, 1) gw_lists_kernel(int Nin, long long T,
         const long long c = w0 / CW + h;
         if (c < nch) {
             ws.count[b * nch + c] = (uint32_t)quads | (uint32_t)total << 16;
-            if (!fits) ws.flag[1] = 1u;
+            if (!fits) ws.flag[2] = 1u;
         }
     }
     if (__syncthreads_or(!fits)) return;  // the flag is set: none of this call's lists is read
@@ -264,7 +268,7 @@ __device__ __forceinline__ void sts128(uint32_t a, float2 x, float2 y) {
 
 template <bool VEC>  // g_I rows in 16-byte units
 __global__ void __launch_bounds__(THREADS, 1) gw_sums_kernel(const Args A) {
-    if (__ldg(A.ws.flag + 1)) return;
+    if (too_dense(A.ws.flag)) return;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int q = lane >> 3, l8 = lane & 7;
@@ -400,7 +404,7 @@ __global__ void __launch_bounds__(THREADS, 1) gw_sums_kernel(const Args A) {
 // g_W[i][j] and g_bias[i]: the ranges' sums in order.  32 inputs x 32 neurons per block.
 __global__ void __launch_bounds__(1024) gw_join_kernel(long long N, int Nin, int tiles, int ranges, const Work ws, float *gW,
                                                       float *gb) {
-    if (__ldg(ws.flag + 1)) return;
+    if (too_dense(ws.flag)) return;
     __shared__ float out[NT][33];
     const int x = threadIdx.x, y = threadIdx.y, j0 = blockIdx.x * 32, tile = blockIdx.y;
     const long long stride = (long long)tiles * Nin * NT;
@@ -464,8 +468,8 @@ size_t syn_grad_weights_ws(long long B, long long Nin, long long N, long long T)
     return layout(units, tiles, ranges_for(tiles, units, sms), (int)Nin, nullptr, nullptr);
 }
 
-// g_W and g_bias of a sparse raster; *flags (device): flags[1] set where it is too dense for the
-// lists: then nothing was written, and the caller's other kernel has to run.
+// g_W and g_bias of a sparse raster; *flags (device): flags[1] or flags[2] set where it is too dense for
+// the lists: then nothing was written, and the caller's other kernel has to run.
 int launch_syn_grad_weights(long long B, long long Nin, long long N, long long T, const uint32_t *S, const float *gI,
                             float *gW, float *gb, void *work, const uint32_t **flags, cudaStream_t st) {
     using namespace gwl;
