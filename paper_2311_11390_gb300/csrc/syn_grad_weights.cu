@@ -401,12 +401,13 @@ __global__ void __launch_bounds__(THREADS, 1) gw_sums_kernel(const Args A) {
     }
 }
 
-// g_W[i][j] and g_bias[i]: the ranges' sums in order.  32 inputs x 32 neurons per block.
+// g_W[i][j] and g_bias[i]: the ranges' sums in order.  32 inputs x 32 neurons per block; the neurons' tiles, of which
+// there may be more than 65535, in blockIdx.x.
 __global__ void __launch_bounds__(1024) gw_join_kernel(long long N, int Nin, int tiles, int ranges, const Work ws, float *gW,
                                                       float *gb) {
     if (too_dense(ws.flag)) return;
     __shared__ float out[NT][33];
-    const int x = threadIdx.x, y = threadIdx.y, j0 = blockIdx.x * 32, tile = blockIdx.y;
+    const int x = threadIdx.x, y = threadIdx.y, j0 = blockIdx.y * 32, tile = blockIdx.x;
     const long long stride = (long long)tiles * Nin * NT;
     if (gW) {
         float s = 0.0f;
@@ -420,7 +421,7 @@ __global__ void __launch_bounds__(1024) gw_join_kernel(long long N, int Nin, int
         const long long i = (long long)tile * NT + y;
         if (i < N && j0 + x < Nin) gW[i * Nin + j0 + x] = out[y][x];
     }
-    if (gb && blockIdx.x == 0 && y == 0) {
+    if (gb && blockIdx.y == 0 && y == 0) {
         const long long i = (long long)tile * NT + x;
         float s = 0.0f;
         for (int r = 0; r < ranges; ++r) s += ws.part_b[((long long)r * tiles + tile) * NT + x];
@@ -493,7 +494,7 @@ int launch_syn_grad_weights(long long B, long long Nin, long long N, long long T
     sums<<<(unsigned)(A.tiles * A.ranges), THREADS, smem_of((int)Nin), st>>>(A);
     e = cudaGetLastError();
     if (e != cudaSuccess) return (int)e;
-    gw_join_kernel<<<dim3((unsigned)((Nin + 31) / 32), (unsigned)A.tiles), dim3(32, 32), 0, st>>>(N, (int)Nin, A.tiles,
+    gw_join_kernel<<<dim3((unsigned)A.tiles, (unsigned)((Nin + 31) / 32)), dim3(32, 32), 0, st>>>(N, (int)Nin, A.tiles,
                                                                                               A.ranges, A.ws, gW, gb);
     return (int)cudaGetLastError();
 }
