@@ -183,7 +183,9 @@ __global__ void __launch_bounds__(TH_MAX, 2) vr_forward_kernel(long long T, cons
         }
 #pragma unroll
         for (int k = 0; k < WORD / 2; ++k) s[k & 1] = __ffma2_rn(f[k], f[k], s[k & 1]);
-        acc = df_add(acc, df{(s[0].x + s[0].y) + (s[1].x + s[1].y), 0.0f});
+        // FP32 sums of 8 squares, joined without rounding
+        const df u = two_sum(s[0].x, s[0].y), v = two_sum(s[1].x, s[1].y), w = two_sum(u.hi, v.hi);
+        acc = df_add(acc, quick_two_sum(w.hi, (u.lo + v.lo) + w.lo));
     }
 #pragma unroll
     for (int off = 16; off; off >>= 1) {
