@@ -157,6 +157,17 @@ def _stream(device=None):
     return torch.cuda.current_stream(device).cuda_stream
 
 
+def _scratch(n: int, device):
+    """n bytes for event lists, which a call can do without: (tensor, n), or (None, 0) where none are
+    used or they no longer fit on the device."""
+    if n > 0:
+        try:
+            return torch.empty(n, dtype=torch.uint8, device=device), n
+        except torch.cuda.OutOfMemoryError:
+            pass
+    return None, 0
+
+
 def _f32(t, shape=None):
     if t is None:
         return None
@@ -449,8 +460,7 @@ def syn_project(S_words: torch.Tensor, W_hi: torch.Tensor, W_lo: torch.Tensor, b
     if out is None:
         out = torch.empty((B, N, T), dtype=torch.float32, device=S_words.device)
     L = lib()
-    wsz = int(L.syn_project_workspace_size(B, Nin, N, T))
-    ws = torch.empty(wsz, dtype=torch.uint8, device=S_words.device) if wsz else None
+    ws, wsz = _scratch(int(L.syn_project_workspace_size(B, Nin, N, T)), S_words.device)
     _check(L.syn_project_ws(B, Nin, N, T, _ptr(W_hi), _ptr(W_lo), ldw, _ptr(S_words), _ptr(bias), _ptr(out),
                             _ptr(ws), wsz, _stream(S_words.device)), "syn_project")
     return out
@@ -467,8 +477,7 @@ def syn_project_backward(S_words, grad_I, W=None, Nin=None, want_gW=True, want_g
     L = lib()
     wsz = int(L.syn_project_backward_workspace_size(B, N, Nin))
     ws = torch.empty(max(wsz, 4), dtype=torch.uint8, device=dev)
-    lsz = int(L.syn_project_backward_lists_size(B, Nin, N, T)) if want_gW or want_gb else 0
-    lists = torch.empty(lsz, dtype=torch.uint8, device=dev) if lsz else None
+    lists, lsz = _scratch(int(L.syn_project_backward_lists_size(B, Nin, N, T)) if want_gW or want_gb else 0, dev)
     _check(L.syn_project_backward_ws(B, Nin, N, T, _ptr(W), _ptr(S_words), _ptr(grad_I), _ptr(gW), _ptr(gS),
                                      _ptr(gb), _ptr(ws), wsz, _ptr(lists), lsz, _stream(dev)), "syn_project_backward")
     return gW, gS, gb
@@ -581,8 +590,7 @@ def syn_project_events(S_words: torch.Tensor, W_t: torch.Tensor, bias=None, Nin=
     if out is None:
         out = torch.empty((B, N, T), dtype=torch.float32, device=S_words.device)
     L = lib()
-    wsz = int(L.syn_project_events_workspace_size(B, Nin, N, T))
-    ws = torch.empty(wsz, dtype=torch.uint8, device=S_words.device) if wsz else None
+    ws, wsz = _scratch(int(L.syn_project_events_workspace_size(B, Nin, N, T)), S_words.device)
     _check(L.syn_project_events_ws(B, Nin, N, T, _ptr(W_t), _ptr(S_words), _ptr(bias), _ptr(out), _ptr(ws), wsz,
                                    _stream(S_words.device)), "syn_project_events")
     return out
