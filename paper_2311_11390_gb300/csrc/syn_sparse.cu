@@ -62,9 +62,12 @@ inline size_t layout(long long tiles, int rec, void *base, Work *w) {
 }
 
 // Starts a workspace's flags: [0] no dense tile yet, [1] whether a sample of the raster has more than
-// `limit` active inputs per step, [2] no list that did not fit (weight gradients).  One block, 4 words per thread (131 000 input steps; 32 words took
-// 30 us: one SM's random reads).
+// `limit` active inputs per step, [2] no list that did not fit (weight gradients).  One block, 4 words per
+// thread (131 000 input steps; 32 words took 30 us: one SM's random reads).  The sampled word of each 4096th
+// of the raster is at a scattered place in it: at equal distances, which were multiples of the words per row
+// for many sizes (128 x 256 x 1000 steps among them), every sample fell on the same 32 steps.
 constexpr int SAMPLE = 4;
+static_assert(1024 * SAMPLE == 1 << 12, "a 4096th per sampled word");
 __global__ void __launch_bounds__(1024, 1) sample_kernel(const uint32_t *__restrict__ S, long long words, long long Nin,
                                                          float limit, uint32_t *flags) {
     __shared__ int part[32];
@@ -73,8 +76,13 @@ __global__ void __launch_bounds__(1024, 1) sample_kernel(const uint32_t *__restr
     uint32_t v[SAMPLE];
 #pragma unroll
     for (int m = 0; m < SAMPLE; ++m) {
-        const long long k = m * 1024 + tid;
-        v[m] = k < n ? __ldg(S + k * words / n) : 0u;  // n <= 2^12 and words < 2^45: no overflow
+        const uint32_t k = m * 1024 + tid;
+        uint32_t h = k * 2654435769u;  // scattered over 32 bits (odd multipliers and shifted exclusive-ors)
+        h = (h ^ h >> 15) * 2246822519u;
+        h ^= h >> 13;
+        // floor((k + h / 2^32) words / 4096) < words
+        const uint64_t at = words > n ? __umul64hi(((uint64_t)k << 32 | h) << 20, (uint64_t)words) : k;
+        v[m] = k < n ? __ldg(S + at) : 0u;
     }
     int c = 0;
 #pragma unroll
