@@ -478,10 +478,11 @@ int syn_project_backward(int64_t B, int64_t Nin, int64_t N, int64_t T, const flo
 
 /* syn_project_backward() with a second workspace for event lists (256-byte aligned,
  * syn_project_backward_lists_size() bytes; 0 where it is not used): grad_W and grad_bias of sparse
- * rasters (at Nin = 1000 up to 8 spikes per step on average and in every 512 steps) are then summed
- * from lists built once for all neurons, each weight's spikes in the order of the steps within 512
- * steps and those sums in the order of time, in a fixed number of ranges (deterministic on a given
- * GPU model).  Denser rasters, and calls with lists = NULL, run as syn_project_backward(). */
+ * rasters (at Nin = 1000 up to 10 spikes per step on average) are then summed from lists built once
+ * for all neurons, each weight's spikes in the order of the steps within 512 steps (read from the
+ * raster where 512 steps hold more than the list does) and those sums in the order of time, in a fixed
+ * number of ranges (deterministic on a given GPU model).  Denser rasters, and calls with lists = NULL,
+ * run as syn_project_backward(). */
 size_t syn_project_backward_lists_size(int64_t B, int64_t Nin, int64_t N, int64_t T);
 int syn_project_backward_ws(int64_t B, int64_t Nin, int64_t N, int64_t T, const float *W,
                             const uint32_t *S_in, const float *grad_I, float *grad_W,

@@ -12,6 +12,9 @@
 //     serves four spikes without bank conflicts (8 lanes read one 128-byte row) and the warp never
 //     diverges; then the four inputs' sums are updated.  The next unit's g_I (registers) and lists
 //     (cp.async, double-buffered) are on their way meanwhile.
+//     A unit with more spikes than its list holds is walked from the raster instead (walk_unit): at
+//     64 x 512 -> 512 x 4096 steps with one such unit per batch element 0.35 ms, where the whole call
+//     went to the other kernel 0.55.
 //   * gw_join_kernel adds the ranges' sums in a fixed order: deterministic.
 // What bounds it: shared-memory traffic.  Per spike and 32 neurons its 128-byte column is read and, at
 // 1000 inputs, 30 Hz and 0.1 ms, another 128 bytes of sums are (an input's sums are read and written
@@ -51,9 +54,9 @@ __host__ __device__ constexpr int rec_of(int Nin) { return HEAD + 16 * rows_of(N
 __host__ __device__ constexpr int smem_of(int Nin) { return GT_BYTES + sums_bytes(Nin) + 2 * rec_of(Nin) + 64; }
 static_assert(smem_of(MAX_NIN) <= SMEM && rows_of(MAX_NIN) >= 1000, "10 spikes a step fit at any Nin");
 
-// Workspace: [1] whether a sample of the raster is too dense for the lists, [2] whether a unit's list
-// did not fit (two words: the lists kernel, whose blocks all decide by [1] whether to run, writes [2]);
-// from byte 256 the units' sizes (groups | rows << 16), their records, the ranges' sums [range][tile][input][32] and of g_I itself [range][tile][32].
+// Workspace: [1] whether a sample of the raster is too dense for the lists (written by the sample alone);
+// from byte 256 the units' sizes (groups | rows << 16, or OVER for one whose list does not fit), their
+// records, the ranges' sums [range][tile][input][32] and of g_I itself [range][tile][32].
 struct Work {
     uint32_t *flag, *count;
     unsigned char *rec;
@@ -84,8 +87,7 @@ inline int ranges_for(long long tiles, long long units, int sms) {
     return best;
 }
 
-// Whether the other kernel has to run: after the lists kernel, when nobody writes the flags any more.
-__device__ __forceinline__ bool too_dense(const uint32_t *flag) { return __ldg(flag + 1) | __ldg(flag + 2); }
+constexpr uint32_t OVER = 0xffffu;
 
 // One CTA per 1024 steps (two units) of a batch element: a warp holds a 32nd of the rows, a lane the
 // word of 32 steps, so that the raster is read in whole lines.
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(1024, 1) gw_lists_kernel(int Nin, long long T,
     __shared__ uint16_t count[2][MAX_NIN], slot[2][MAX_NIN], order[2][MAX_NIN];
     __shared__ int bin[2][BINS];
     __shared__ int upto[2][MAX_QUADS], warp_rows[2][8];
+    __shared__ bool fit[2];
     const int rec = rec_of(Nin), cap = rows_of(Nin);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int half = lane >> 4, l16 = lane & 15;
@@ -208,11 +211,11 @@ __global__ void __launch_bounds__(1024, 1) gw_lists_kernel(int Nin, long long T,
     if (tid == 0 || tid == 512) {
         const long long c = w0 / CW + h;
         if (c < nch) {
-            ws.count[b * nch + c] = (uint32_t)quads | (uint32_t)total << 16;
-            if (!fits) ws.flag[2] = 1u;
+            ws.count[b * nch + c] = fits ? (uint32_t)quads | (uint32_t)total << 16 : OVER;
         }
+        fit[h] = fits;
     }
-    if (__syncthreads_or(!fits)) return;  // the flag is set: none of this call's lists is read
+    __syncthreads();
     // the steps
 #pragma unroll
     for (int m = 0; m < 32; ++m) {
@@ -227,7 +230,7 @@ __global__ void __launch_bounds__(1024, 1) gw_lists_kernel(int Nin, long long T,
             if (l16 >= l) e += o;
         }
         e -= c;  // this word's first spike among the input's
-        if (y) {
+        if (y && fit[half]) {
             const int s = slot[half][row];
             uint16_t *to = reinterpret_cast<uint16_t *>(recs + half * rec + HEAD + 16 * (upto[half][s >> 2] + 1)) + 2 * (s & 3);
             while (y) {
@@ -239,7 +242,7 @@ __global__ void __launch_bounds__(1024, 1) gw_lists_kernel(int Nin, long long T,
     }
     __syncthreads();
     const long long c = w0 / CW + h;
-    if (c < nch) {
+    if (c < nch && fits) {
         uint4 *to = reinterpret_cast<uint4 *>(ws.rec + (b * nch + c) * rec);
         for (int k = i; k < HEAD / 16 + total; k += 512) to[k] = reinterpret_cast<const uint4 *>(record)[k];
     }
@@ -249,6 +252,7 @@ struct Args {
     long long N, T, nch, units;
     int Nin, tiles, ranges, rec;
     const float *gI;
+    const uint32_t *S;
     Work ws;
 };
 
@@ -266,9 +270,40 @@ __device__ __forceinline__ void sts128(uint32_t a, float2 x, float2 y) {
     asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(x.x), "f"(x.y), "f"(y.x), "f"(y.y) : "memory");
 }
 
+// The sums of a unit whose list does not fit, from the raster: 8 lanes take an input, two of its 16 words
+// each, and walk its spikes together; the same additions in the same order as from a list.
+__device__ __noinline__ void walk_unit(const Args &A, long long u, uint32_t gt, uint32_t sums) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, q = lane >> 3, l8 = lane & 7;
+    const long long nwin = (A.T + 31) / 32, b = u / A.nch, w0 = (u - b * A.nch) * CW + 2 * l8;
+    const uint32_t gl = gt + 16 * l8, tail = (A.T & 31) ? (1u << (A.T & 31)) - 1u : ~0u;
+    for (int j0 = 4 * warp; j0 < A.Nin; j0 += 4 * WARPS) {
+        const int j = j0 + q;
+        const uint32_t *row = A.S + (b * A.Nin + j) * nwin;
+        uint32_t v[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            v[k] = j < A.Nin && w0 + k < nwin ? __ldg(row + w0 + k) : 0u;
+            if (w0 + k == nwin - 1) v[k] &= tail;
+        }
+        const uint32_t p = sums + (j < A.Nin ? j : A.Nin) * (NT * 4) + 16 * l8;  // the row past the last: scratch
+        float2 a0 = make_float2(0.0f, 0.0f), a1 = a0;
+        for (int k = 0; k < CW; ++k) {
+            uint32_t m = __shfl_sync(FULL, (k & 1) ? v[1] : v[0], (lane & 24) | k >> 1);
+            while (__any_sync(FULL, m != 0u)) {
+                const float4 x = lds128(gl + 16 * (m ? row_of(32 * k + __ffs(m) - 1) : ZERO_ROW));
+                m &= m - 1u;
+                a0 = __fadd2_rn(a0, make_float2(x.x, x.y));
+                a1 = __fadd2_rn(a1, make_float2(x.z, x.w));
+            }
+        }
+        const float4 s = lds128(p);
+        sts128(p, __fadd2_rn(a0, make_float2(s.x, s.y)), __fadd2_rn(a1, make_float2(s.z, s.w)));
+    }
+}
+
 template <bool VEC>  // g_I rows in 16-byte units
-__global__ void __launch_bounds__(THREADS, 1) gw_sums_kernel(const Args A) {
-    if (too_dense(A.ws.flag)) return;
+__global__ void __launch_bounds__(THREADS, 1) gw_sums_kernel(const __grid_constant__ Args A) {
+    if (__ldg(A.ws.flag + 1)) return;
     extern __shared__ __align__(128) unsigned char smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int q = lane >> 3, l8 = lane & 7;
@@ -348,7 +383,9 @@ __global__ void __launch_bounds__(THREADS, 1) gw_sums_kernel(const Args A) {
         const uint32_t rec = lists + half * A.rec, gl = gt + 16 * l8;
         const int quads = (int)(size & 0xffffu);
         size = count_now;
-        if (warp < quads) {
+        if (quads == (int)OVER) {
+            walk_unit(A, u, gt, sums);
+        } else if (warp < quads) {
             uint32_t at;
             asm volatile("ld.shared.u16 %0, [%1];" : "=r"(at) : "r"(rec + 2 * warp));
             const uint32_t row0 = rec + HEAD + 4 * q;
@@ -405,7 +442,7 @@ __global__ void __launch_bounds__(THREADS, 1) gw_sums_kernel(const Args A) {
 // there may be more than 65535, in blockIdx.x.
 __global__ void __launch_bounds__(1024) gw_join_kernel(long long N, int Nin, int tiles, int ranges, const Work ws, float *gW,
                                                       float *gb) {
-    if (too_dense(ws.flag)) return;
+    if (__ldg(ws.flag + 1)) return;
     __shared__ float out[NT][33];
     const int x = threadIdx.x, y = threadIdx.y, j0 = blockIdx.y * 32, tile = blockIdx.x;
     const long long stride = (long long)tiles * Nin * NT;
@@ -469,13 +506,13 @@ size_t syn_grad_weights_ws(long long B, long long Nin, long long N, long long T)
     return layout(units, tiles, ranges_for(tiles, units, sms), (int)Nin, nullptr, nullptr);
 }
 
-// g_W and g_bias of a sparse raster; *flags (device): flags[1] or flags[2] set where it is too dense for
-// the lists: then nothing was written, and the caller's other kernel has to run.
+// g_W and g_bias of a sparse raster; *flags (device): flags[1] set where it is too dense for the
+// lists: then nothing was written, and the caller's other kernel has to run.
 int launch_syn_grad_weights(long long B, long long Nin, long long N, long long T, const uint32_t *S, const float *gI,
                             float *gW, float *gb, void *work, const uint32_t **flags, cudaStream_t st) {
     using namespace gwl;
     const long long nwin = (T + 31) / 32, nch = (T + CH - 1) / CH;
-    Args A{N, T, nch, B * nch, (int)Nin, (int)((N + NT - 1) / NT), 1, rec_of((int)Nin), gI, {}};
+    Args A{N, T, nch, B * nch, (int)Nin, (int)((N + NT - 1) / NT), 1, rec_of((int)Nin), gI, S, {}};
     const int sms = sm_count();
     if (!sms) return (int)cudaErrorInvalidDevice;
     A.ranges = ranges_for(A.tiles, A.units, sms);

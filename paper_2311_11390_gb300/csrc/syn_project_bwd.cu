@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(LTHREADS, 1) gw_lane_kernel(const float *__res
                                                               const uint32_t *__restrict__ S, long long N,
                                                               long long Nin, long long T, int nwin, int ldp,
                                                               float *part, float *part_b, const uint32_t *flags) {
-    if (flags && !(__ldg(flags + 1) | __ldg(flags + 2))) return;  // the list path has computed everything
+    if (flags && !__ldg(flags + 1)) return;  // the list path has computed everything
     extern __shared__ float sm[];
     float *gt = sm;                                                          // [LCH][LGS]
     uint32_t *wsl = reinterpret_cast<uint32_t *>(sm + (size_t)LCH * LGS);   // [2][LTHREADS][LCW] word slots
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(LTHREADS, 1) gw_lane_kernel(const float *__res
 // Fixed-order sum over the batch: g_W[i][j] = sum_b part[b][i][j]; g_bias[i] likewise.
 __global__ void gw_reduce_kernel(const float *part, const float *part_b, long long B, long long N, long long Nin,
                                  int ldp, float *gW, float *gb, const uint32_t *flags) {
-    if (flags && !(__ldg(flags + 1) | __ldg(flags + 2))) return;
+    if (flags && !__ldg(flags + 1)) return;
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < N * Nin) {
         const long long i = k / Nin, j = k % Nin;

@@ -62,7 +62,7 @@ inline size_t layout(long long tiles, int rec, void *base, Work *w) {
 }
 
 // Starts a workspace's flags: [0] no dense tile yet, [1] whether a sample of the raster has more than
-// `limit` active inputs per step, [2] no list that did not fit (weight gradients).  One block, 4 words per
+// `limit` active inputs per step.  One block, 4 words per
 // thread (131 000 input steps; 32 words took 30 us: one SM's random reads).  The sampled word of each 4096th
 // of the raster is at a scattered place in it: at equal distances, which were multiples of the words per row
 // for many sizes (128 x 256 x 1000 steps among them), every sample fell on the same 32 steps.
@@ -95,7 +95,6 @@ __global__ void __launch_bounds__(1024, 1) sample_kernel(const uint32_t *__restr
         if (lane == 0) {
             flags[0] = 0u;
             flags[1] = (float)c * (float)Nin > limit * 32.0f * (float)n;
-            flags[2] = 0u;
         }
     }
 }
