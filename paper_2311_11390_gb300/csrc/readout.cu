@@ -24,38 +24,54 @@ __device__ __forceinline__ float warp_sum(float x) {
     return x;
 }
 
-// n[b,k] = sum_t w[t] S[b,k,t] and o[b,c] = sum_k W[c,k] n[b,k] + bias_c w_sum: one block per batch
-// element, a warp per row, lanes over its words, then a warp per output, lanes over the inputs.  Bound by
-// latency: with a kernel for each sum and a thread per output 27 us at B = 128, K = 256, C = 20, T = 1000,
-// now 13.
-__global__ void forward_kernel(long long K, long long C, long long T, long long nwords, const uint32_t *__restrict__ S,
-                               const float *__restrict__ w, const float *__restrict__ W,
-                               const float *__restrict__ bias, float w_sum, float *n, float *o) {
-    const long long b = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    float *nb = n + b * K;
-    for (long long k = warp; k < K; k += nwarp) {
-        const uint32_t *row = S + (b * K + k) * nwords;
-        float acc = 0.0f;
-        for (long long q = lane; q < nwords; q += 32) {
-            uint32_t word = __ldg(row + q);
-            if (q == nwords - 1 && (T & 31)) word &= (1u << (T & 31)) - 1u;
-            while (word) {
-                const int i = __ffs(word) - 1;
-                word &= word - 1u;
-                acc += __ldg(w + q * 32 + i);
-            }
+// n[r] = sum_t w[t] S[r,t] of one row: lanes over its words, four of them loaded together.
+__device__ __forceinline__ float count_row(const uint32_t *__restrict__ row, long long T, long long nwords,
+                                           const float *__restrict__ w, int lane) {
+    float acc = 0.0f;
+    for (long long q0 = lane; q0 < nwords; q0 += 128) {
+        uint32_t v[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            const long long q = q0 + 32 * m;
+            v[m] = q < nwords ? __ldg(row + q) : 0u;
+            if (q == nwords - 1 && (T & 31)) v[m] &= (1u << (T & 31)) - 1u;
         }
-        acc = warp_sum(acc);
-        if (lane == 0) nb[k] = acc;
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+            while (v[m]) {
+                const int i = __ffs(v[m]) - 1;
+                v[m] &= v[m] - 1u;
+                acc += __ldg(w + (q0 + 32 * m) * 32 + i);
+            }
     }
-    __syncthreads();
-    for (long long c = warp; c < C; c += nwarp) {
-        float acc = 0.0f;
-        for (long long k = lane; k < K; k += 32) acc = fmaf(__ldg(W + c * K + k), nb[k], acc);
-        acc = warp_sum(acc);
-        if (lane == 0) o[b * C + c] = bias ? fmaf(bias[c], w_sum, acc) : acc;
-    }
+    return warp_sum(acc);
+}
+
+// n[b,k]: a warp per row, over the whole grid.  Bound by the raster's latency: at 128 x 1024 rows of 16000 steps
+// 220 us with one load of a word in flight per lane, 86 (with out_kernel) with four.
+__global__ void __launch_bounds__(256) count_kernel(long long rows, long long T, long long nwords,
+                                                    const uint32_t *__restrict__ S, const float *__restrict__ w, float *n) {
+    const long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (r >= rows) return;
+    const float acc = count_row(S + r * nwords, T, nwords, w, threadIdx.x & 31);
+    if ((threadIdx.x & 31) == 0) n[r] = acc;
+}
+
+// o[b,c] = sum_k W[c,k] n[b,k] + bias_c w_sum: a warp per output, lanes over the inputs (a thread per output
+// walked 1024 inputs in 35 us).  Counts and outputs in one launch, a block per batch element, measured no less
+// anywhere and far more where a block's rows are many or long (us, this / that): 128 x 256 x 1000 steps 9.9 / 11,
+// 1 x 256 x 1000 5.0 / 10, 32 x 1024 x 16000 28 / 117, 1 x 1024 x 16000 11 / 109.
+__global__ void __launch_bounds__(256) out_kernel(long long BC, long long K, long long C, const float *__restrict__ W,
+                                                  const float *__restrict__ bias, float w_sum,
+                                                  const float *__restrict__ n, float *o) {
+    const long long e = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (e >= BC) return;
+    const long long b = e / C, c = e - b * C;
+    float acc = 0.0f;
+    for (long long k = lane; k < K; k += 32) acc = fmaf(__ldg(W + c * K + k), __ldg(n + b * K + k), acc);
+    acc = warp_sum(acc);
+    if (lane == 0) o[e] = bias ? fmaf(bias[c], w_sum, acc) : acc;
 }
 
 // dL/dS[r, t] = w[t] h[r], h[b,k] = sum_c W[c,k] g_o[b,c]: one warp per row r = (b, k).
@@ -163,9 +179,17 @@ __global__ void pack_kernel(long long rows, long long T, long long nwords, const
 
 int launch_readout_forward(long long B, long long K, long long C, long long T, const uint32_t *S, const float *W,
                            const float *bias, const float *w, float w_sum, float *n, float *o, cudaStream_t st) {
-    if (B <= 0) return 0;
-    ro::forward_kernel<<<(unsigned)B, 1024, 0, st>>>(K, C, T, (T + 31) / 32, S, w, W, bias, w_sum, n, o);
-    return (int)cudaGetLastError();
+    const long long rows = B * K;
+    if (rows > 0) {
+        ro::count_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(rows, T, (T + 31) / 32, S, w, n);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return (int)e;
+    }
+    if (B * C > 0) {
+        ro::out_kernel<<<(unsigned)((B * C + 7) / 8), 256, 0, st>>>(B * C, K, C, W, bias, w_sum, n, o);
+        return (int)cudaGetLastError();
+    }
+    return 0;
 }
 
 int launch_readout_backward(long long B, long long K, long long C, long long T, const float *W, const float *w,
