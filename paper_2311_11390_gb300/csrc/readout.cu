@@ -74,23 +74,32 @@ __global__ void __launch_bounds__(256) out_kernel(long long BC, long long K, lon
     if (lane == 0) o[e] = bias ? fmaf(bias[c], w_sum, acc) : acc;
 }
 
-// dL/dS[r, t] = w[t] h[r], h[b,k] = sum_c W[c,k] g_o[b,c]: one warp per row r = (b, k).
-__device__ __forceinline__ void grad_spikes(long long r, int lane, long long K, long long C, long long T,
-                                            const float *__restrict__ W, const float *__restrict__ g_o,
+// dL/dS[r, t] = w[t] h[r], h[b,k] = sum_c W[c,k] g_o[b,c]: one warp per row r = (b, k) and steps t0 .. t1 - 1.
+// Loads go out together, of h's chain (10 per step of the loop) and of w before the stores (which could alias it
+// for all the compiler knows).
+__device__ __forceinline__ void grad_spikes(long long r, long long t0, long long t1, int lane, long long K, long long C,
+                                            long long T, const float *__restrict__ W, const float *__restrict__ g_o,
                                             const float *__restrict__ w, float *gS) {
     const long long b = r / K, k = r % K;
     float h = 0.0f;
-#pragma unroll 4
+#pragma unroll 10
     for (long long c = 0; c < C; ++c) h = fmaf(__ldg(W + c * K + k), __ldg(g_o + b * C + c), h);
     float *out = gS + r * T;
     if ((T & 3) == 0 && ((reinterpret_cast<uintptr_t>(gS) & 15u) == 0) &&
         ((reinterpret_cast<uintptr_t>(w) & 15u) == 0)) {
-        for (long long t = 4LL * lane; t < T; t += 128) {
-            const float4 wv = *reinterpret_cast<const float4 *>(w + t);
-            *reinterpret_cast<float4 *>(out + t) = make_float4(h * wv.x, h * wv.y, h * wv.z, h * wv.w);
+        constexpr int U = 4;
+        for (long long t = t0 + 4 * lane; t < t1; t += 128 * U) {
+            float4 v[U];
+#pragma unroll
+            for (int m = 0; m < U; ++m)
+                if (t + 128 * m < t1) v[m] = __ldg(reinterpret_cast<const float4 *>(w + t + 128 * m));
+#pragma unroll
+            for (int m = 0; m < U; ++m)
+                if (t + 128 * m < t1)
+                    *reinterpret_cast<float4 *>(out + t + 128 * m) = make_float4(h * v[m].x, h * v[m].y, h * v[m].z, h * v[m].w);
         }
     } else {
-        for (long long t = lane; t < T; t += 32) out[t] = h * w[t];
+        for (long long t = t0 + lane; t < t1; t += 32) out[t] = h * __ldg(w + t);
     }
 }
 
@@ -113,18 +122,27 @@ __device__ __forceinline__ void grad_w(long long e, long long B, long long K, lo
     }
 }
 
+constexpr long long WARPS = 32 * 152;  // that fill the chip with writes
+
 // Both gradients in one launch: the first nw blocks take grad_w's elements (a serial sum over the batch,
-// hidden behind the writes of the others), the rest grad_spikes' rows.  As two kernels 27 + 30 us at
-// B = 128, K = 256, C = 20, T = 1000, now 37 (the 131 MB written take 19).
-__global__ void __launch_bounds__(256, 8) backward_kernel(unsigned nw, long long B, long long K, long long C, long long T,
-                                const float *__restrict__ W, const float *__restrict__ g_o,
-                                const float *__restrict__ w, const float *__restrict__ n, float w_sum, float *gS,
-                                float *gW, float *gb) {
+// hidden behind the writes of the others), the rest grad_spikes' rows in `parts` parts of `len` steps.  Bound by the
+// writes of dL/dS: at B = 128, K = 256, C = 20, T = 1000 (131 MB) 24 us, as two kernels, with a load at a time,
+// 55; at 128 x 1024 x 16000 1.13 ms and 1.17.
+__global__ void __launch_bounds__(256, 4) backward_kernel(unsigned nw, long long B, long long K, long long C, long long T,
+                                long long parts, long long len, const float *__restrict__ W,
+                                const float *__restrict__ g_o, const float *__restrict__ w,
+                                const float *__restrict__ n, float w_sum, float *gS, float *gW, float *gb) {
     if (blockIdx.x < nw) {
         grad_w((long long)blockIdx.x * blockDim.x + threadIdx.x, B, K, C, g_o, n, w_sum, gW, gb);
     } else {
-        const long long r = (long long)(blockIdx.x - nw) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-        if (r < B * K) grad_spikes(r, threadIdx.x & 31, K, C, T, W, g_o, w, gS);
+        long long r = (long long)(blockIdx.x - nw) * (blockDim.x >> 5) + (threadIdx.x >> 5), t0 = 0;
+        if (parts > 1) {
+            const long long q = r / parts;
+            t0 = (r - q * parts) * len;
+            r = q;
+        }
+        const long long t1 = t0 + len < T ? t0 + len : T;
+        if (r < B * K && t0 < T) grad_spikes(r, t0, t1, threadIdx.x & 31, K, C, T, W, g_o, w, gS);
     }
 }
 
@@ -198,9 +216,16 @@ int launch_readout_backward(long long B, long long K, long long C, long long T, 
     const long long m = gW && C * K > C ? C * K : C;
     const unsigned nw = (gW || gb) && m > 0 ? (unsigned)((m + 255) / 256) : 0;
     const long long rows = gS && T > 0 ? B * K : 0;
-    const unsigned ns = (unsigned)((rows + 7) / 8);
+    // few rows are cut into parts of at least 512 steps, so that some 32 warps per SM write (1 x 1024 x 16000:
+    // 13 us, 22 with a warp per row)
+    long long parts = 1, len = T;
+    if (rows > 0 && rows < ro::WARPS) {
+        parts = ro::WARPS / rows < (T + 511) / 512 ? ro::WARPS / rows : (T + 511) / 512;
+        len = ((T + parts - 1) / parts + 127) / 128 * 128;
+    }
+    const unsigned ns = (unsigned)((rows * parts + 7) / 8);
     if (nw + ns == 0) return 0;
-    ro::backward_kernel<<<nw + ns, 256, 0, st>>>(nw, B, K, C, T, W, g_o, w, n, w_sum, gS, gW, gb);
+    ro::backward_kernel<<<nw + ns, 256, 0, st>>>(nw, B, K, C, T, parts, len, W, g_o, w, n, w_sum, gS, gW, gb);
     return (int)cudaGetLastError();
 }
 
