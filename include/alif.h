@@ -145,7 +145,7 @@ int64_t alif_ckpt_count(int64_t T);
  *   ckpt     [B,N,alif_ckpt_count(T)] AlifState: state entering step 256k, or NULL
  *            (alif_backward needs it)
  *   final_state [B,N] AlifState state entering step T, or NULL
- * With B*N >= 80 x the SM count (and no traces), a lane takes a row and walks
+ * With B*N >= 80 x the SM count, or 32 x it and 45 T (and no traces), a lane takes a row and walks
  * it through Blocks of K <= T_eff steps (K = 16, 8 or 4; below, step by step): the Block's
  * no-reset membrane (Prop 1) from an input-only chain, its first crossing
  * (Prop 2, Eq 9), and the state carried to the next Block (Props 3-5).  With
@@ -203,7 +203,7 @@ int alif_forward_window(int steps);
 
 /* Layout of alif_forward (host; a performance choice: the spikes are the same,
  * checkpoints and final states agree within FP32 rounding).  0, the default: a
- * lane per row when B * N >= 80 x the SM count, a warp per row otherwise.
+ * lane per row when B * N >= 80 x the SM count, or 32 x it and 45 T, a warp per row otherwise.
  * 1: a warp per row (the windows above).  2: a lane per row: each lane walks its
  * row through Blocks of K <= T_R steps (K = 16, 8 or 4 by the smallest T_eff of
  * the warp's 32 rows; step by step below 4), at most one spike per Block (Section 3.1), with the

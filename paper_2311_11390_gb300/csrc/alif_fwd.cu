@@ -917,8 +917,12 @@ int launch_alif_forward(long long B, long long N, long long T, const float *I,
     // it declines calls it cannot stage with TMA.  Its time hardly depends on the rows up to 32768, the
     // warp-per-row kernel's is proportional to them; 2000 steps, us, lanes / warps at 8192, 12288 and
     // 16384 rows: T_eff = 20 66 / 49, 69 / 66, 68 / 80; 10 76 / 50, 78 / 64, 78 / 81; 4 146 / 102,
-    // 146 / 146, 148 / 175; 2 109 / 103, 109 / 149, 109 / 175
-    const bool lanes = g_fwd_layout == 2 || (g_fwd_layout == 0 && A.rows >= 80LL * g_sm_count);
+    // 146 / 146, 148 / 175; 2 109 / 103, 109 / 149, 109 / 175.  A warp's window costs its 256 steps however few
+    // there are, so from 32 rows per SM on short rows go to lanes: 5000 rows of 100 steps (T_eff 20, 4) 7 / 11, 11 / 12,
+    // 8192 of 160 9 / 13, 15 / 16, 12100 of 256 12 / 18, 23 / 25; not 4864 of 160 7 / 11, 15 / 12, 8192 of 256 12 / 13, 24 / 18
+    const bool lanes = g_fwd_layout == 2 ||
+                       (g_fwd_layout == 0 && (A.rows >= 80LL * g_sm_count ||
+                                              (A.rows >= 32LL * g_sm_count && 45 * T <= A.rows)));
     if (lanes && !vtr && !atr) {
         bool declined = false;
         const int rc =
