@@ -71,11 +71,14 @@ inline size_t layout(long long units, long long tiles, int ranges, int Nin, void
     return o4 + (size_t)ranges * tiles * NT * 4;
 }
 
-// Ranges of units per neuron tile: the fewest for which the CTAs fill whole waves to 6 %.
+// Ranges of units per neuron tile: the fewest for which the CTAs fill whole waves to 6 %, out of 64 or, where the
+// tiles are one or two, as many as fill the SMs (with 64 CTAs for one tile 249 x 186 -> 16 x 4105 steps took 138 us,
+// now 115).
 inline int ranges_for(long long tiles, long long units, int sms) {
     int best = 1;
     double least = 1e30;
-    for (int p = 1; p <= 64 && p <= units; ++p) {
+    const long long most = sms / tiles > 64 ? sms / tiles : 64;
+    for (int p = 1; p <= most && p <= units; ++p) {
         const long long ctas = tiles * p;
         const double waste = (double)((ctas + sms - 1) / sms * sms) / (double)ctas;
         if (waste < least - 1e-9) {
@@ -498,7 +501,15 @@ size_t syn_grad_weights_ws(long long B, long long Nin, long long N, long long T)
     if (!sms) return 0;
     const double ctas = (double)B * (double)((N + 15) / 16) * (double)((Nin + 1023) / 1024);
     const double least = active_limit((int)Nin) >= 0.035f * (float)Nin ? 12.0 : 36.0;
-    const bool many = std::ceil(ctas / sms) * (double)((T + 511) / 512) >= least;
+    // Of few neurons the building of the lists is a large part of the work, so the two paths' times are set against each
+    // other as well (us; a wave of the other kernel 9 and 5 per chunk; here 30, for 1024 steps of a batch element
+    // 0.02 + 0.12 per 1000 inputs, for a unit 2 + 2.3): N, that / this as measured 12 60 / 80, 16 95 / 115, 10 104 / 113,
+    // 32 53 / 64, 64 66 / 74 are left to it, and 4 98 / 89, 8 87 / 69, 15 142 / 100, 24 114 / 100, 60 80 / 72 not.
+    const double waves = std::ceil(ctas / sms), chunks = (double)((T + 511) / 512);
+    const double that = waves * (9.0 + 5.0 * chunks);
+    const double here = 30.0 + (double)B * (double)((T + 1023) / 1024) * (0.02 + 0.00012 * (double)Nin) +
+                        std::ceil((double)B * chunks * (double)((N + NT - 1) / NT) / sms) * (2.0 + 0.0023 * (double)Nin);
+    const bool many = waves * chunks >= least && that >= 1.03 * here;
     const double wide = Nin > 350 ? Nin / 350.0 : 1.0;
     if (!many && (double)B * (double)Nin * (double)N * (double)T < 8e9 * wide) return 0;
     const long long units = B * ((T + CH - 1) / CH), tiles = (N + NT - 1) / NT;
