@@ -109,7 +109,9 @@ __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args
     int *pos = reinterpret_cast<int *>(smem + C::ACC_BYTES + (size_t)MAX_EVENTS * 2);  // [GROUPS][32] first slots
     int *off = pos + GROUPS * 32;                                                  // [33] first event of step t
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // units are chunks; with a list, a tile's eight in order (those past T are passed over)
+    // units are chunks; with a list, a tile's eight (those past T are passed over), from another one on for each tile.
+    // In the same order for all they met a grid that is a multiple of 8: of rows of 20 steps, one chunk a tile,
+    // every eighth CTA had all (1873 us at 1000 x 1000 -> 1024 x 20 steps and 20 active inputs, now 400; 263 without lists).
     const uint32_t *dense = LIST && !__ldg(A.dense + 1) ? A.dense + 64 : nullptr;
     const long long units = LIST && dense ? 8LL * __ldg(A.dense) : A.B * A.nwords;
     const long long tiles_t = (A.nwords + 7) / 8;
@@ -129,7 +131,7 @@ __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args
             if (LIST && dense) {
                 const long long tile = __ldg(dense + (u >> 3));
                 b = tile / tiles_t;
-                c = (tile - b * tiles_t) * 8 + (u & 7);
+                c = (tile - b * tiles_t) * 8 + ((u + (u >> 3) + (u >> 6)) & 7);
                 if (c >= A.nwords) continue;
             }
             const int nt = (int)(A.T - c * 32 < 32 ? A.T - c * 32 : 32);  // steps in this chunk
