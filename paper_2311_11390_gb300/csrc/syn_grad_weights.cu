@@ -481,7 +481,8 @@ inline int sm_count() {
 
 }  // namespace gwl
 
-int launch_density_sample(const uint32_t *S, long long words, long long Nin, float limit, uint32_t *flags, cudaStream_t st);
+int launch_density_sample(const uint32_t *S, long long rows, long long Nin, long long T, float limit, uint32_t *flags,
+                          cudaStream_t st);
 
 // Workspace bytes of the list path; 0 where it is not used.
 size_t syn_grad_weights_ws(long long B, long long Nin, long long N, long long T) {
@@ -529,7 +530,7 @@ int launch_syn_grad_weights(long long B, long long Nin, long long N, long long T
     A.ranges = ranges_for(A.tiles, A.units, sms);
     layout(A.units, A.tiles, A.ranges, (int)Nin, work, &A.ws);
     *flags = A.ws.flag;
-    int rc = launch_density_sample(S, B * Nin * nwin, Nin, active_limit((int)Nin), A.ws.flag, st);
+    int rc = launch_density_sample(S, B * Nin, Nin, T, active_limit((int)Nin), A.ws.flag, st);
     if (rc) return rc;
     cudaError_t e = cudaFuncSetAttribute(gw_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (HEAD + 16 * MAX_ROWS));
     if (e != cudaSuccess) return (int)e;

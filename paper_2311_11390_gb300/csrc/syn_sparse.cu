@@ -450,9 +450,12 @@ __global__ void __launch_bounds__(THREADS, 1) sums_kernel(const __grid_constant_
 
 }  // namespace sparse
 
-int launch_density_sample(const uint32_t *S, long long words, long long Nin, float limit, uint32_t *flags,
+// Sample of a raster of `rows` rows (batch elements x inputs): whether more than `limit` of Nin inputs are active per step.
+int launch_density_sample(const uint32_t *S, long long rows, long long Nin, long long T, float limit, uint32_t *flags,
                           cudaStream_t st) {
-    sparse::sample_kernel<<<1, 1024, 0, st>>>(S, words, Nin, limit, flags);
+    const long long nwin = (T + 31) / 32;
+    // the rows' last words hold T % 32 steps: of rows of 20 steps 20 active inputs counted as 12.5
+    sparse::sample_kernel<<<1, 1024, 0, st>>>(S, rows * nwin, Nin, limit * (float)((double)T / (32.0 * (double)nwin)), flags);
     return (int)cudaGetLastError();
 }
 
@@ -499,7 +502,7 @@ int launch_syn_sparse(long long B, long long Nin, long long N, long long T, cons
     // at 9 of 1000, 3.11 against 1.37 at 15 of 512), so there only the records' capacity counts.
     const float room = cap_of((int)Nin) / 32.0f, even = 0.0214f * Nin - 4.5f;
     const float limit = !hi || even > room ? room : even > 6.5f ? even : 6.5f;
-    const int rc = launch_density_sample(S, B * Nin * A.nch, Nin, limit, A.ws.ndense, st);
+    const int rc = launch_density_sample(S, B * Nin, Nin, T, limit, A.ws.ndense, st);
     if (rc) return rc;
     CUtensorMap out = {};
     const bool tma = make_batch_rows_map(&out, I, B, N, T) == 0;
