@@ -20,6 +20,8 @@
 // within (k + 1) 2^-24 (|bias_i| + sum_j |W_ij| S_j) of the exact sum for k active inputs.
 #include <cuda_bf16.h>
 
+#include <cmath>
+
 #include "common.cuh"
 #include "tmap.h"
 
@@ -500,7 +502,10 @@ int launch_syn_sparse(long long B, long long Nin, long long N, long long T, cons
     // 1.5 of 512, 0.65 at 4.6 (0.84): about 0.58 + 0.13 per active input ps an output, against 2.78 Nin /
     // 1000 but no less than 1.43.  The event kernel without lists is slower at every density (2.23 ms
     // at 9 of 1000, 3.11 against 1.37 at 15 of 512), so there only the records' capacity counts.
-    const float room = cap_of((int)Nin) / 32.0f, even = 0.0214f * Nin - 4.5f;
+    // Padded to pairs and to the longest of four, Poisson counts take about a square root more room than their mean: at
+    // 1000 inputs (room for 14 a step) 3 % of the 256-step tiles are over at 9, 59 % at 10, all at 11.  us of the event
+    // projection without / with lists, 32 x 1000 -> 1024 x 4000 steps: 575 / 283, 613 / 522, 655 / 701, and at 12 698 / 736.
+    const float fit = cap_of((int)Nin) / 32.0f, room = fit - 0.95f * sqrtf(fit), even = 0.0214f * Nin - 4.5f;
     const float limit = !hi || even > room ? room : even > 6.5f ? even : 6.5f;
     const int rc = launch_density_sample(S, B * Nin, Nin, T, limit, A.ws.ndense, st);
     if (rc) return rc;

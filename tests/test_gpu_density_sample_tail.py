@@ -21,3 +21,20 @@ def test_steps_of_the_last_word(T, n, dense):
     assert L.syn_project_events_ws(B, Nin, N, T, p(Wt), p(words), None, p(I), p(ws), size, torch.cuda.current_stream().cuda_stream) == 0
     assert int(ws[4:8].view(torch.int32)) == dense
     assert torch.equal(I, S.sum(1, dtype=torch.int32).float()[:, None].expand(B, N, T))  # whole numbers: exact
+
+
+@cuda
+@pytest.mark.parametrize("Nin, n, dense", [(1000, 8, False), (1000, 12, True), (512, 22, False), (512, 27, True)])
+def test_rasters_that_overfill_the_lists(Nin, n, dense):
+    """Counts spread about their mean: the lists hold 14 (30 at 512 inputs) with the padding, not on average."""
+    from paper_2311_11390_gb300 import alif
+    L, p = alif.lib(), lambda t: t.data_ptr()
+    B, N, T = 32, 64, 4000
+    words = alif.pack_spikes((torch.rand((B, Nin, T), device="cuda", generator=torch.Generator(device="cuda").manual_seed(n)) < n / Nin).float())
+    Wt, I = torch.ones((Nin, N), device="cuda"), torch.empty((B, N, T), device="cuda")
+    size = int(L.syn_project_events_workspace_size(B, Nin, N, T))
+    assert size > 0
+    ws = torch.zeros(size, dtype=torch.uint8, device="cuda")
+    assert L.syn_project_events_ws(B, Nin, N, T, p(Wt), p(words), None, p(I), p(ws), size, torch.cuda.current_stream().cuda_stream) == 0
+    assert int(ws[4:8].view(torch.int32)) == dense
+    assert dense or int(ws[:4].view(torch.int32)) < B * ((T + 255) // 256) // 4  # most tiles by lists
