@@ -465,19 +465,21 @@ int launch_density_sample(const uint32_t *S, long long rows, long long Nin, long
 // holds, or a product too small to pay for the lists and three more launches.
 //   * In place of the tensor cores: from 6e10 products on.  There (B = 16, 512 -> 1024, T = 8000) the
 //     dense product takes 0.34 ms and this path about half of it at up to 1.5 active inputs a step;
-//     a raster that turns out dense costs the sample and the empty launches, 15 us, whatever the size.
+//     a raster that turns out dense costs the sample and the empty launches, 8 us, whatever the size.
 //   * In place of the event kernel without lists: from 2e10 (8, 1000 -> 1024, 4000: 72 against
 //     79 us at 1.5 active inputs a step, 78 against 96 at 3).  That kernel's time goes with the 32-step
 //     chunks, about 30 us + 35 ns each whatever N up to 1024, this path's is about 35 us + 0.03 ns a chunk
 //     and neuron, so smaller products too where the chunks are many for the neurons (us, that / this):
 //     27, 512 -> 154, 1800 84 / 41; 10, 700 -> 256, 2001 68 / 42 and at 21 active inputs a step 205 / 68;
 //     32, 128 -> 128, 4000 152 / 42; 7, 512 -> 607, 5100 61 / 54; not for 4, 300 -> 200, 3000 29 / 33 and
-//     1, 512 -> 600, 16000 35 / 37.
+//     1, 512 -> 600, 16000 35 / 37.  A CTA of the lists kernel takes 30 ns
+//     however few of its 1024 steps there are, so not for rows of one chunk either: 2048, 64 -> 64, 32 68 / 93 and 512,
+//     700 -> 256, 32 37 / 44 (64 steps: 128 / 96 and 63 / 48).
 size_t syn_sparse_ws(long long B, long long Nin, long long N, long long T, bool split) {
     using namespace sparse;
     if (B <= 0 || Nin <= 0 || N <= 0 || T <= 0 || Nin > MAX_NIN) return 0;
     const double chunks = (double)B * (double)((T + 31) / 32);
-    const bool many = !split && chunks * (1150.0 - (double)N) >= 4e5;
+    const bool many = !split && T > 32 && chunks * (1150.0 - (double)N) >= 4e5;
     if (!many && (double)B * (double)Nin * (double)N * (double)T < (split ? 6e10 : 2e10)) return 0;
     const long long tiles = B * ((T + TILE - 1) / TILE);
     if (tiles > (1LL << 30) || (N + NT - 1) / NT > (1LL << 30)) return 0;
