@@ -502,19 +502,21 @@ int launch_alif_forward_recurrent(long long B, long long N, long long T, int TR,
     for (int nbuf = 2; nbuf >= 1 && !found; --nbuf)
         for (int wch = MAX_WCH; wch >= 4 && !found; wch /= 2) found = fits(vw, pitch_of(TR, vw), nbuf, wch);
     if (!found && !fits(1, TR, 1, 4)) return -1;
-    const size_t smem = smem_bytes(A);
-    auto kern = per <= 256 ? (vw == 4   ? rec_fwd_kernel<256, 4>
-                              : vw == 2 ? rec_fwd_kernel<256, 2>
-                                        : rec_fwd_kernel<256, 1>)
-                           : (vw == 4   ? rec_fwd_kernel<MAX_PER, 4>
-                              : vw == 2 ? rec_fwd_kernel<MAX_PER, 2>
-                                        : rec_fwd_kernel<MAX_PER, 1>);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const auto kern = per <= 256 ? (vw == 4   ? rec_fwd_kernel<256, 4>
+                                    : vw == 2 ? rec_fwd_kernel<256, 2>
+                                              : rec_fwd_kernel<256, 1>)
+                                 : (vw == 4   ? rec_fwd_kernel<MAX_PER, 4>
+                                    : vw == 2 ? rec_fwd_kernel<MAX_PER, 2>
+                                              : rec_fwd_kernel<MAX_PER, 1>);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(A));
+    if (e != cudaSuccess) return (int)e;
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return (int)e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(B * G), 1, 1);
     cfg.blockDim = dim3((unsigned)per, 1, 1);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = smem_bytes(A);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -523,6 +525,27 @@ int launch_alif_forward_recurrent(long long B, long long N, long long T, int TR,
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (2 * B * G > sms && A.wch > 32) {
+        // More clusters than may fit at a time (with a CTA per SM): a wave less is worth more than slots (32 x 1024 x
+        // 1000 at T_R = 60: 64 slots, a CTA per SM, 779 us; 32 slots, two, 322).
+        long long least = 0;
+        int best = 0;
+        for (int wch = A.wch; wch >= 32; wch /= 2) {
+            fits(vw, A.P, A.nbuf, wch);
+            cfg.dynamicSmemBytes = smem_bytes(A);
+            int n = 0;
+            e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+            if (e != cudaSuccess) return (int)e;
+            const long long waves = (B + n - 1) / (n > 0 ? n : 1);
+            if (best == 0 || waves < least) {
+                least = waves;
+                best = wch;
+            }
+            if (waves == 1) break;
+        }
+        fits(vw, A.P, A.nbuf, best);
+        cfg.dynamicSmemBytes = smem_bytes(A);
+    }
     e = cudaLaunchKernelEx(&cfg, kern, A);
     return (int)e;
 }
