@@ -106,10 +106,11 @@ __device__ __forceinline__ void cp_async_wait() {
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// MAXT: the CTA size the register budget is sized for (256: up to 255 registers a thread, for
-// clusters of at most 256 neurons per CTA; 1024 otherwise).  VW: floats per unit of the currents.
-template <int MAXT, int VW>
-__global__ void __launch_bounds__(MAXT, 1) rec_fwd_kernel(const Args A) {
+// MAXT, MINB: the CTA size and the CTAs per SM the register budget is sized for (256, 1: up to 255
+// registers a thread, for clusters of at most 256 neurons per CTA; 256, 2: up to 128).  VW: floats per unit of
+// the currents.
+template <int MAXT, int MINB, int VW>
+__global__ void __launch_bounds__(MAXT, MINB) rec_fwd_kernel(const Args A) {
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char smem[];
     const int per = A.per, TR = A.TR, G = A.G, nbuf = A.nbuf, wch = A.wch;
@@ -502,14 +503,13 @@ int launch_alif_forward_recurrent(long long B, long long N, long long T, int TR,
     for (int nbuf = 2; nbuf >= 1 && !found; --nbuf)
         for (int wch = MAX_WCH; wch >= 4 && !found; wch /= 2) found = fits(vw, pitch_of(TR, vw), nbuf, wch);
     if (!found && !fits(1, TR, 1, 4)) return -1;
-    const auto kern = per <= 256 ? (vw == 4   ? rec_fwd_kernel<256, 4>
-                                    : vw == 2 ? rec_fwd_kernel<256, 2>
-                                              : rec_fwd_kernel<256, 1>)
-                                 : (vw == 4   ? rec_fwd_kernel<MAX_PER, 4>
-                                    : vw == 2 ? rec_fwd_kernel<MAX_PER, 2>
-                                              : rec_fwd_kernel<MAX_PER, 1>);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(A));
-    if (e != cudaSuccess) return (int)e;
+    using Kernel = void (*)(Args);
+    const auto kernel = [&](bool pairs) -> Kernel {
+        if (per > 256) return vw == 4 ? rec_fwd_kernel<MAX_PER, 1, 4> : vw == 2 ? rec_fwd_kernel<MAX_PER, 1, 2> : rec_fwd_kernel<MAX_PER, 1, 1>;
+        if (pairs) return vw == 4 ? rec_fwd_kernel<256, 2, 4> : vw == 2 ? rec_fwd_kernel<256, 2, 2> : rec_fwd_kernel<256, 2, 1>;
+        return vw == 4 ? rec_fwd_kernel<256, 1, 4> : vw == 2 ? rec_fwd_kernel<256, 1, 2> : rec_fwd_kernel<256, 1, 1>;
+    };
+    Kernel kern = kernel(false);
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return (int)e;
@@ -525,27 +525,37 @@ int launch_alif_forward_recurrent(long long B, long long N, long long T, int TR,
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (2 * B * G > sms && A.wch > 32) {
-        // More clusters than may fit at a time (with a CTA per SM): a wave less is worth more than slots (32 x 1024 x
-        // 1000 at T_R = 60: 64 slots, a CTA per SM, 779 us; 32 slots, two, 322).
+    if (2 * B * G > sms) {
+        // More clusters than may fit at a time with a CTA per SM: a wave less is worth more than slots (32 x 1024 x 1000
+        // at T_R = 60: 64 slots, a CTA per SM, 779 us; 32 slots, two, 322) and than registers (of more than 192 neurons a
+        // CTA two need 128 a thread: 32 x 2000 x 300 at T_R = 20 232 us with one, 125 with two).
         long long least = 0;
-        int best = 0;
-        for (int wch = A.wch; wch >= 32; wch /= 2) {
-            fits(vw, A.P, A.nbuf, wch);
-            cfg.dynamicSmemBytes = smem_bytes(A);
-            int n = 0;
-            e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+        int slots = 0;
+        bool two = false;
+        const int most = A.wch;
+        for (int pairs = 0; pairs <= (per > 192 && per <= 256) && least != 1; ++pairs) {
+            e = cudaFuncSetAttribute(kernel(pairs), cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
             if (e != cudaSuccess) return (int)e;
-            const long long waves = (B + n - 1) / (n > 0 ? n : 1);
-            if (best == 0 || waves < least) {
-                least = waves;
-                best = wch;
+            for (int wch = most; wch >= (most < 32 ? most : 32) && least != 1; wch /= 2) {
+                fits(vw, A.P, A.nbuf, wch);
+                cfg.dynamicSmemBytes = smem_bytes(A);
+                int n = 0;
+                e = cudaOccupancyMaxActiveClusters(&n, kernel(pairs), &cfg);
+                if (e != cudaSuccess) return (int)e;
+                const long long waves = (B + n - 1) / (n > 0 ? n : 1);
+                if (least == 0 || waves < least) {
+                    least = waves;
+                    slots = wch;
+                    two = pairs;
+                }
             }
-            if (waves == 1) break;
         }
-        fits(vw, A.P, A.nbuf, best);
+        fits(vw, A.P, A.nbuf, slots);
         cfg.dynamicSmemBytes = smem_bytes(A);
+        kern = kernel(two);
     }
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);  // one value for all threads
+    if (e != cudaSuccess) return (int)e;
     e = cudaLaunchKernelEx(&cfg, kern, A);
     return (int)e;
 }

@@ -32,3 +32,21 @@ def test_long_blocks_of_many_clusters():
     for k in ("spikes", "I_total", "final"):  # and the slots change no bit
         assert torch.equal(outs[0][k], outs[1][k][:8])
     assert times[1] < 1.8 * times[0], times
+
+
+@cuda
+def test_two_ctas_of_256_neurons():
+    """2000 neurons: CTAs of 256, two to an SM where clusters are many; the bits of few clusters."""
+    from paper_2311_11390_gb300 import alif
+    N, T = 2000, 300
+    g = torch.Generator(device="cuda").manual_seed(7)
+    u = lambda lo, hi: (lo + (hi - lo) * torch.rand(N, generator=g, device="cuda")).cpu().numpy()  # noqa: E731
+    table = alif.neuron_table(u(10, 30), u(100, 500), u(1, 1), u(0, 0.2), dt_ms=0.1, arp_ms=2.0)
+    I = 1.2 + 0.5 * torch.randn((32, N, T), generator=g, device="cuda")
+    W = alif.transpose_weights(0.5 * torch.randn((N, N), generator=g, device="cuda") / N ** 0.5)
+    for length in (300, 298, 297):  # units of 4, 2 and 1 steps
+        x = I[..., :length].contiguous()
+        many, few = alif.forward_recurrent(x, W, table, 0.1, 2.0), alif.forward_recurrent(x[:2].contiguous(), W, table, 0.1, 2.0)
+        assert alif.device_status() == 0
+        for k in ("spikes", "I_total", "final", "ckpt"):
+            assert torch.equal(many[k][:2], few[k])
