@@ -49,7 +49,7 @@ namespace rec {
 constexpr int MAX_G = 8;           // portable cluster size
 constexpr int MAX_PER = 1024;      // neurons per CTA
 constexpr int NO_SPIKE = -1;
-constexpr int MAX_WCH = 64;        // recurrent weights copied together
+constexpr int MAX_WCH = 128;       // recurrent weights copied together
 constexpr uint32_t NO_STEP = 1023;  // step of the entries past the last spike (T_R <= 1023)
 
 struct Args {
@@ -105,6 +105,41 @@ __device__ __forceinline__ void cp_async_wait() {
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// Sums of a chunk's weights, sorted by step, into a neuron's currents: event k's weight is w0, the next one's w1, ev2 the
+// entry after.
+template <int VW>
+struct Events {
+    const float *wcol;
+    const uint32_t *p;
+    int per;
+    uint32_t ev0, ev1, ev2;
+    float w0, w1;
+    __device__ __forceinline__ void start(const float *w, const uint32_t *sorted, int n) {
+        wcol = w;
+        per = n;
+        ev0 = sorted[0];
+        ev1 = sorted[1];
+        ev2 = sorted[2];
+        p = sorted + 3;
+        w0 = wcol[(ev0 >> 10) * per];
+        w1 = wcol[(ev1 >> 10) * per];
+    }
+    __device__ __forceinline__ void add(int u, Vec<VW> &I, Vec<VW> &lo) {  // steps u .. u + VW - 1
+#pragma unroll
+        for (int s = 0; s < VW; ++s)
+            while ((int)(ev0 & 1023u) == u + s) {  // the same spikes in every thread of the CTA
+                const df s2 = two_sum(I.v[s], w0);
+                I.v[s] = s2.hi;
+                lo.v[s] += s2.lo;
+                ev0 = ev1;
+                w0 = w1;
+                ev1 = ev2;
+                w1 = wcol[(ev1 >> 10) * per];
+                ev2 = *p++;  // at most the fourth entry past the last spike's
+            }
+    }
+};
 
 // MAXT, MINB: the CTA size and the CTAs per SM the register budget is sized for (256, 1: up to 255
 // registers a thread, for clusters of at most 256 neurons per CTA; 256, 2: up to 128).  VW: floats per unit of
@@ -242,19 +277,49 @@ __global__ void __launch_bounds__(MAXT, MINB) rec_fwd_kernel(const Args A) {
             }
             cp_async_commit();
         };
+        auto sort_chunk = [&](int e0, int nch) {  // by step, and within one in the order of the list
+            for (int e = tid; e < nch; e += per) {
+                const uint32_t mine = (list[e0 + e] & 1023u) << 7 | (uint32_t)e;
+                int at = 0;
+#pragma unroll 8
+                for (int o = 0; o < nch; ++o) at += ((list[e0 + o] & 1023u) << 7 | (uint32_t)o) < mine;
+                sorted[at] = (uint32_t)e << 10 | mine >> 7;
+            }
+            if (tid < 4) sorted[nch + tid] = NO_STEP;
+        };
         int e0 = 0;
         const bool multi = total > wch;
-        for (; total - e0 > wch; e0 += wch) {  // more spikes than weight slots: added into the buffers
+        // More spikes than weight slots: all but the last few are added into the buffers beforehand.  Of up to 256 neurons
+        // a CTA each spike by itself; above, where the step's places of a warp's neurons meet in eight banks, a chunk
+        // sorted and summed like the last one (2 x 4096 x 400 steps at 130 spikes a Block 537 -> 383 us; 16 x 2000 x 500
+        // at 78 432 against 405, but 32 x 1024 x 1000 at T_R = 60 322 against 341, and 2 % on T_R = 2 and 10 without any
+        // such chunk).
+        for (; total - e0 > wch; e0 += wch) {
             copy_weights(e0, wch);
+            if constexpr (MAXT > 256) sort_chunk(e0, wch);
             cp_async_wait<0>();
             __syncthreads();
-            if (live)
-                for (int k = 0; k < wch; ++k) {
-                    const int at = tid * P + (int)(list[e0 + k] & 1023u);
-                    const df s2 = two_sum(cur[at], wbuf[(size_t)k * per + tid]);
-                    cur[at] = s2.hi;
-                    acl[at] += s2.lo;
+            if (live) {
+                if constexpr (MAXT > 256) {
+                    float *mycur = cur + tid * P, *mylo = acl + tid * P;
+                    Events<VW> ev;
+                    ev.start(wbuf + tid, sorted, per);
+                    for (int u = 0; u < cnt; u += VW) {
+                        if ((int)(ev.ev0 & 1023u) >= u + VW) continue;
+                        Vec<VW> I = *reinterpret_cast<const Vec<VW> *>(mycur + u), lo = *reinterpret_cast<const Vec<VW> *>(mylo + u);
+                        ev.add(u, I, lo);
+                        *reinterpret_cast<Vec<VW> *>(mycur + u) = I;
+                        *reinterpret_cast<Vec<VW> *>(mylo + u) = lo;
+                    }
+                } else {
+                    for (int k = 0; k < wch; ++k) {
+                        const int at = tid * P + (int)(list[e0 + k] & 1023u);
+                        const df s2 = two_sum(cur[at], wbuf[(size_t)k * per + tid]);
+                        cur[at] = s2.hi;
+                        acl[at] += s2.lo;
+                    }
                 }
+            }
             __syncthreads();
         }
         const int nch = total - e0;
@@ -264,14 +329,7 @@ __global__ void __launch_bounds__(MAXT, MINB) rec_fwd_kernel(const Args A) {
             load_ff(n + 1);
             cp_async_commit();
         }
-        for (int e = tid; e < nch; e += per) {  // by step, and within one in the order of the list
-            const uint32_t mine = (list[e0 + e] & 1023u) << 6 | (uint32_t)e;
-            int at = 0;
-#pragma unroll 8
-            for (int o = 0; o < nch; ++o) at += ((list[e0 + o] & 1023u) << 6 | (uint32_t)o) < mine;
-            sorted[at] = (uint32_t)e << 10 | mine >> 6;
-        }
-        if (tid < 4) sorted[nch + tid] = NO_STEP;
+        sort_chunk(e0, nch);
         if (pref)
             cp_async_wait<1>();
         else
