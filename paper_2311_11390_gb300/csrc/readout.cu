@@ -24,26 +24,34 @@ __device__ __forceinline__ float warp_sum(float x) {
     return x;
 }
 
-// n[r] = sum_t w[t] S[r,t] of one row: lanes over its words, four of them loaded together.
+// Sum of w over the set bits of M words of a row, 32 apart from word q on, loaded together.
+template <int M>
+__device__ __forceinline__ float count_words(const uint32_t *__restrict__ row, long long q, long long T, long long nwords,
+                                             const float *__restrict__ w, float acc) {
+    uint32_t v[M];
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+        v[m] = q + 32 * m < nwords ? __ldg(row + q + 32 * m) : 0u;
+        if (q + 32 * m == nwords - 1 && (T & 31)) v[m] &= (1u << (T & 31)) - 1u;
+    }
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+        while (v[m]) {
+            const int i = __ffs(v[m]) - 1;
+            v[m] &= v[m] - 1u;
+            acc += __ldg(w + (q + 32 * m) * 32 + i);
+        }
+    return acc;
+}
+
+// n[r] = sum_t w[t] S[r,t] of one row: lanes over its words, four at a time where there are more than 32.
 __device__ __forceinline__ float count_row(const uint32_t *__restrict__ row, long long T, long long nwords,
                                            const float *__restrict__ w, int lane) {
     float acc = 0.0f;
-    for (long long q0 = lane; q0 < nwords; q0 += 128) {
-        uint32_t v[4];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const long long q = q0 + 32 * m;
-            v[m] = q < nwords ? __ldg(row + q) : 0u;
-            if (q == nwords - 1 && (T & 31)) v[m] &= (1u << (T & 31)) - 1u;
-        }
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-            while (v[m]) {
-                const int i = __ffs(v[m]) - 1;
-                v[m] &= v[m] - 1u;
-                acc += __ldg(w + (q0 + 32 * m) * 32 + i);
-            }
-    }
+    if (nwords <= 32)
+        acc = count_words<1>(row, lane, T, nwords, w, acc);
+    else
+        for (long long q = lane; q < nwords; q += 128) acc = count_words<4>(row, q, T, nwords, w, acc);
     return warp_sum(acc);
 }
 
