@@ -440,7 +440,7 @@ int syn_project(int64_t B, int64_t Nin, int64_t N, int64_t T,
                 const uint32_t *S_in, const float *bias, float *I, void *stream);
 
 /* syn_project() with a workspace for the event lists of sparse rasters.  256-step tiles whose
- * chunks of 32 steps are sparse enough (at Nin = 1000 about 12 active inputs per step) are summed over
+ * chunks of 32 steps are sparse enough (at Nin = 1000 about 10 active inputs per step) are summed over
  * the active inputs only, with the weights W_hi + W_lo in FP32, inputs ascending and the bias last:
  * within (k + 1) 2^-24 (|bias_i| + sum_j |W_ij| S_j) of the exact sum of W_hi + W_lo for k active
  * inputs.  The other tiles run on the tensor cores as in syn_project().  A weight that is not finite
@@ -478,7 +478,7 @@ int syn_project_backward(int64_t B, int64_t Nin, int64_t N, int64_t T, const flo
 
 /* syn_project_backward() with a second workspace for event lists (256-byte aligned,
  * syn_project_backward_lists_size() bytes; 0 where it is not used): grad_W and grad_bias of sparse
- * rasters (at Nin = 1000 up to 10 spikes per step on average) are then summed from lists built once
+ * rasters (at Nin = 1000 up to 11 spikes per step on average) are then summed from lists built once
  * for all neurons, each weight's spikes in the order of the steps within 512 steps (read from the
  * raster where 512 steps hold more than the list does) and those sums in the order of time, in a fixed
  * number of ranges (deterministic on a given GPU model).  Denser rasters, and calls with lists = NULL,

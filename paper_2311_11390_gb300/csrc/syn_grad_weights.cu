@@ -19,7 +19,7 @@
 // What bounds it: shared-memory traffic.  Per spike and 32 neurons its 128-byte column is read and, at
 // 1000 inputs, 30 Hz and 0.1 ms, another 128 bytes of sums are (an input's sums are read and written
 // once per 512 steps); every staged value is written once.  B = 32, 1000 -> 1024, T = 16000: sums
-// 0.90 ms (events alone 0.48, staging without events 0.47: the two overlap badly, loads or L2
+// 0.86 ms (events alone 0.48, staging without events 0.47: the two overlap badly, loads or L2
 // prefetches issued a unit ahead notwithstanding), lists 0.07, against 2.41 ms for a thread per input
 // that walks its own spikes, whose warps wait for their busiest lane.
 #include "common.cuh"

@@ -14,7 +14,7 @@
 // more than 8 steps.
 // What bounds it: the gradient's writes (4 B per step, 0.24 ms for 1024 rows x 400000 steps; the
 // bits are 1/16 of that) and the instructions of the word's chains and scans between the barriers.
-// At that size: forward 0.14 ms, gradient 0.44 ms.  A warp per row walking 256-step windows left it
+// At that size: forward 0.19 ms, gradient 0.46 ms.  A warp per row walking 256-step windows left it
 // to 1024 warps that each waited for two spike words per window: 0.92 and 2.05 ms.
 #include "common.cuh"
 
