@@ -98,11 +98,19 @@ struct Args {
     const uint32_t *dense;  // NULL or dense[1]: every chunk; else those of dense[0] tiles, listed from dense[64]
 };
 
-// LIST: only the chunks of the tiles listed at A.dense
-template <int NPT, bool LIST>
+// ALL: every chunk.  LISTED: the chunks of the tiles listed at A.dense, or all when dense[1] is set.  One neuron per
+// thread has these two as kernels of their own, ALL_IF and LISTED_IF: with both in one, however it was written, every
+// chunk of a dense raster took 7 to 11 % longer (84 x 942 -> 1023 x 302 steps at 47 active inputs a step 800 us, 730
+// without lists, 739 as two).  From 2e10 products on: below, an empty launch more is a larger part of a sparse raster's
+// call than those are of a dense one's.
+enum Walk { ALL, LISTED, ALL_IF, LISTED_IF };
+template <int NPT, Walk WALK>
 __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args A) {
     using C = Cfg<NPT>;
     constexpr int THREADS = C::THREADS, WARPS = C::WARPS, WPT = C::WPT, ACC_STRIDE = C::ACC_STRIDE;
+    constexpr bool LIST = WALK == LISTED || WALK == LISTED_IF;
+    if (WALK == ALL_IF && !__ldg(A.dense + 1)) return;
+    if (WALK == LISTED_IF && __ldg(A.dense + 1)) return;
     extern __shared__ __align__(16) unsigned char smem[];
     float *acc = reinterpret_cast<float *>(smem);                                  // [32][ACC_STRIDE] step x neuron
     uint16_t *list = reinterpret_cast<uint16_t *>(smem + C::ACC_BYTES);            // [MAX_EVENTS] (t << 10) | input
@@ -112,7 +120,7 @@ __global__ void __launch_bounds__(Cfg<NPT>::THREADS, 1) events_kernel(const Args
     // units are chunks; with a list, a tile's eight (those past T are passed over), from another one on for each tile.
     // In the same order for all they met a grid that is a multiple of 8: of rows of 20 steps, one chunk a tile,
     // every eighth CTA had all (1873 us at 1000 x 1000 -> 1024 x 20 steps and 20 active inputs, now 400; 263 without lists).
-    const uint32_t *dense = LIST && !__ldg(A.dense + 1) ? A.dense + 64 : nullptr;
+    const uint32_t *dense = LIST && (WALK == LISTED_IF || !__ldg(A.dense + 1)) ? A.dense + 64 : nullptr;
     const long long units = LIST && dense ? 8LL * __ldg(A.dense) : A.B * A.nwords;
     const long long tiles_t = (A.nwords + 7) / 8;
     const int nblk = (int)((A.Nin + IN_BLOCK - 1) / IN_BLOCK);
@@ -304,7 +312,7 @@ int launch_syn_project_events(long long B, long long Nin, long long N, long long
     const long long units = B * A.nwords;
     if (units == 0 || N == 0) return 0;
     static int sms = 0;
-    static bool attr[6] = {false, false, false, false, false, false};
+    static bool attr[8] = {};
     if (!sms) {
         int dev = 0;
         cudaGetDevice(&dev);
@@ -325,13 +333,15 @@ int launch_syn_project_events(long long B, long long Nin, long long N, long long
         return (int)cudaGetLastError();
     };
     if (dense) {
-        if (npt == 4) return go(events_kernel<4, true>, Cfg<4>::SMEM_BYTES, Cfg<4>::THREADS, 5);
-        if (npt == 2) return go(events_kernel<2, true>, Cfg<2>::SMEM_BYTES, Cfg<2>::THREADS, 4);
-        return go(events_kernel<1, true>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 3);
+        if (npt == 4) return go(events_kernel<4, LISTED>, Cfg<4>::SMEM_BYTES, Cfg<4>::THREADS, 5);
+        if (npt == 2) return go(events_kernel<2, LISTED>, Cfg<2>::SMEM_BYTES, Cfg<2>::THREADS, 4);
+        if ((double)B * (double)Nin * (double)N * (double)T < 2e10) return go(events_kernel<1, LISTED>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 7);
+        const int rc = go(events_kernel<1, ALL_IF>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 3);
+        return rc ? rc : go(events_kernel<1, LISTED_IF>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 6);
     }
-    if (npt == 4) return go(events_kernel<4, false>, Cfg<4>::SMEM_BYTES, Cfg<4>::THREADS, 2);
-    if (npt == 2) return go(events_kernel<2, false>, Cfg<2>::SMEM_BYTES, Cfg<2>::THREADS, 1);
-    return go(events_kernel<1, false>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 0);
+    if (npt == 4) return go(events_kernel<4, ALL>, Cfg<4>::SMEM_BYTES, Cfg<4>::THREADS, 2);
+    if (npt == 2) return go(events_kernel<2, ALL>, Cfg<2>::SMEM_BYTES, Cfg<2>::THREADS, 1);
+    return go(events_kernel<1, ALL>, Cfg<1>::SMEM_BYTES, Cfg<1>::THREADS, 0);
 }
 
 }  // namespace alif
